@@ -381,7 +381,8 @@ def _sparse(sc, views, n, g):
         u, w = (place[at, 0] * (W - 1)).round().long(), (place[at, 1] * (H - 1)).round().long()
         pix = torch.stack([u.double(), w.double(), torch.ones_like(u).double()], 1)
         d = views[v][1][w, u, 3].double()
-        X[at] = (d[:, None] * (pix @ torch.linalg.inv(K).T) - t) @ R
+        Kinv = torch.as_tensor(np.linalg.inv(sc.cams[v][0]), device=DEV)
+        X[at] = (d[:, None] * (pix @ Kinv.T) - t) @ R
     vis = torch.zeros(n, dtype=torch.int64, device=DEV)
     obs = torch.full((n, 2), math.nan, dtype=torch.float64, device=DEV)
     for v, (K, R, t) in enumerate(cams):
