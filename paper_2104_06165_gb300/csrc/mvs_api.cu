@@ -43,6 +43,8 @@ struct BatchGraph {
     std::vector<int32_t> refs, srcs;
     mvs_pm_params params;
     int lanes = 0;
+    const float4* draws = nullptr; // workspace the kernels were captured with
+    const float* win = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long kernels = 0;
     unsigned long long used = 0;   // call counter of the last use (least recently used is replaced)
@@ -54,7 +56,7 @@ struct mvs_ctx {
     cudaStream_t stream = nullptr;
     std::vector<ViewData> views;
     std::string err;
-    Scratch scratch[8];
+    Scratch scratch[9];
     // measurement hooks
     bool prof = false;
     std::vector<cudaEvent_t> ev;
@@ -250,6 +252,33 @@ mvs_status ensure_map(mvs_ctx* c, int32_t v) {
     return MVS_OK;
 }
 
+// The phases' workspace, one per context (its views run one after another):
+// the refinement perturbations of an iteration (20 bytes per pixel), then, when
+// the call visits every pixel often enough to pay for storing the windows (an
+// initialisation, which builds them anyway, or at least two iterations) and
+// they take at most kWindowBytes, the stored windows; otherwise the phases
+// rebuild each window, with the same results.
+constexpr size_t kWindowBytes = (size_t)16 << 30;
+cudaError_t use_workspace(mvs_ctx* c, RefConst& rc, size_t max_pixels, const mvs_pm_params* p, int phases) {
+    if (phases == 0) return cudaSuccess;
+    const bool init = p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE;
+    const size_t draws = (max_pixels * 20 + 255) & ~(size_t)255;
+    size_t windows = phases >= (init ? 1 : 4) ? max_pixels * pm_window_bytes(rc) : 0;
+    if (windows > kWindowBytes) windows = 0;
+    cudaError_t e;
+    char* b = (char*)scratch(c, 8, draws + windows, &e);
+    if (e != cudaSuccess && windows) {   // no room for the windows
+        cudaGetLastError();
+        windows = 0;
+        b = (char*)scratch(c, 8, draws, &e);
+    }
+    if (e != cudaSuccess) return e;
+    rc.draw4 = (float4*)b;
+    rc.draw1 = (float*)(b + max_pixels * 16);
+    rc.win = windows ? (float*)(b + draws) : nullptr;
+    return cudaSuccess;
+}
+
 // fills n floats with v
 __global__ void k_fill(float* __restrict__ a, size_t n, float v) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) a[i] = v;
@@ -369,8 +398,11 @@ mvs_status mvs_patchmatch(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t 
     size_t n = (size_t)V.cam.width * V.cam.height;
     RefConst rc;
     make_refconst(c, ref, srcs, n_src, p, rc);
-    if (p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE) {
-        CK(c, launch_init(rc, nullptr, c->stream));
+    const bool init = p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE;
+    CK(c, use_workspace(c, rc, n, p, pend - p->phase_begin));
+    if (rc.win && !init) CK(c, launch_windows(rc, c->stream));
+    if (init) {
+        CK(c, launch_init(rc, c->stream));
     } else {
         CK(c, cudaMemcpyAsync(V.plane, out->plane, n * sizeof(float4), kind_in(out->mem), c->stream));
         if (p->init_mode == MVS_INIT_GIVEN)
@@ -390,7 +422,7 @@ mvs_status mvs_patchmatch(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t 
             }
             CK(c, cudaEventRecord(c->ev[c->ev_used], c->stream));
         }
-        CK(c, launch_phase(rcp, ph, c->stream));
+        CK(c, launch_phase(rcp, ph, ph == p->phase_begin, c->stream));
         if (c->prof) {
             CK(c, cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
             c->ev_used += 2;
@@ -428,7 +460,7 @@ static mvs_status autotune_lanes(mvs_ctx* c, int32_t ref, const int32_t* srcs, i
     cudaError_t e;
     char* keep = (char*)scratch(c, 5, n * (sizeof(float4) + sizeof(float)), &e);
     CK(c, e);
-    CK(c, launch_init(rc, nullptr, c->stream));
+    CK(c, launch_init(rc, c->stream));
     CK(c, cudaMemcpyAsync(keep, V.plane, n * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream));
     CK(c, cudaMemcpyAsync(keep + n * sizeof(float4), V.cost, n * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
     cudaEvent_t t0, t1;
@@ -438,13 +470,15 @@ static mvs_status autotune_lanes(mvs_ctx* c, int32_t ref, const int32_t* srcs, i
     int best = cand[0];
     for (int lanes : cand) {
         rc.lanes_hint = lanes;
+        CK(c, use_workspace(c, rc, n, &q, 4));   // the stored windows follow the layout
+        if (rc.win) CK(c, launch_windows(rc, c->stream));
         for (int rep = 0; rep < 2; ++rep) {   // the first run warms caches and launch configuration
             CK(c, cudaMemcpyAsync(V.plane, keep, n * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream));
             CK(c, cudaMemcpyAsync(V.cost, keep + n * sizeof(float4), n * sizeof(float), cudaMemcpyDeviceToDevice,
                                   c->stream));
             CK(c, cudaEventRecord(t0, c->stream));
             CK(c, launch_memo_reset(rc, c->stream));
-            for (int ph = 0; ph < 4; ++ph) CK(c, launch_phase(rc, ph, c->stream));
+            for (int ph = 0; ph < 4; ++ph) CK(c, launch_phase(rc, ph, ph == 0, c->stream));
             CK(c, cudaEventRecord(t1, c->stream));
         }
         CK(c, cudaEventSynchronize(t1));
@@ -513,12 +547,15 @@ mvs_status mvs_patchmatch_batch(mvs_ctx* c, int32_t n_ref, const int32_t* refs, 
             prop_off += (size_t)rcs[r].W * rcs[r].H * rcs[r].n_prop;
         }
     }
+    size_t most = 0;
+    for (auto& rc : rcs) most = std::max(most, (size_t)rc.W * rc.H);
+    for (auto& rc : rcs) CK(c, use_workspace(c, rc, most, p, pend - p->phase_begin));
     std::vector<int32_t> kr(refs, refs + n_ref), ks(srcs, srcs + (size_t)n_ref * n_src);
     // a graph captured for the same call, else the least recently used slot
     BatchGraph* hit = nullptr;
     BatchGraph* lru = &c->batch[0];
     for (auto& b : c->batch) {
-        if (b.exec && b.refs == kr && b.srcs == ks && b.lanes == q.lanes_per_pixel &&
+        if (b.exec && b.refs == kr && b.srcs == ks && b.lanes == q.lanes_per_pixel && b.draws == rcs[0].draw4 && b.win == rcs[0].win &&
             std::memcmp(&b.params, &q, sizeof q) == 0)
             hit = &b;
         if (!b.exec || (lru->exec && b.used < lru->used)) lru = &b;
@@ -535,12 +572,15 @@ mvs_status mvs_patchmatch_batch(mvs_ctx* c, int32_t n_ref, const int32_t* refs, 
         cudaError_t e = cudaSuccess;
         // view after view: consecutive launches share their source textures in L2
         for (int r = 0; r < n_ref && e == cudaSuccess; ++r) {
-            if (p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE)
-                e = launch_init(rcs[r], nullptr, c->gstream);
+            const bool init = p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE;
+            if (rcs[r].win && !init) e = launch_windows(rcs[r], c->gstream);
+            if (e != cudaSuccess) break;
+            if (init)
+                e = launch_init(rcs[r], c->gstream);
             else if (p->init_mode == MVS_INIT_GIVEN_RECOST)
                 e = launch_cost(rcs[r], rcs[r].plane, rcs[r].cost, nullptr, c->gstream);
             if (e == cudaSuccess) e = launch_memo_reset(rcs[r], c->gstream);
-            for (int ph = p->phase_begin; ph < pend && e == cudaSuccess; ++ph) e = launch_phase(rcs[r], ph, c->gstream);
+            for (int ph = p->phase_begin; ph < pend && e == cudaSuccess; ++ph) e = launch_phase(rcs[r], ph, ph == p->phase_begin, c->gstream);
         }
         cudaError_t e2 = cudaStreamEndCapture(c->gstream, &g);
         if (e == cudaSuccess) e = e2;
@@ -553,6 +593,8 @@ mvs_status mvs_patchmatch_batch(mvs_ctx* c, int32_t n_ref, const int32_t* refs, 
         B.srcs = ks;
         B.params = q;
         B.lanes = q.lanes_per_pixel;
+        B.draws = rcs[0].draw4;
+        B.win = rcs[0].win;
     }
     // order the private stream after the caller's stream, replay, and back
     CK(c, cudaEventRecord(c->gev[0], c->stream));

@@ -65,6 +65,9 @@ struct RefConst {
     int precision;             // 0 = FP32, 1 = mixed (half2 bilinear, FP32 moments)
     int n_prop;                // learned proposals per pixel (0 = none)
     const float4* props;       // H*W*n_prop planes (n, depth), or null
+    float* win;                // stored windows (win_record_floats per pixel), or null: rebuilt at each visit
+    float4* draw4;             // refinement perturbations of the current iteration, per pixel: delta_d,
+    float* draw1;              // cos / sin delta_theta, cos delta_phi | sin delta_phi
     const float2* init_range;  // H*W (d_min, d_max) of the sparse-feature initialisation (NaN: none), or null
     PairConst pair[MVS_MAX_SRC];
 };
@@ -115,9 +118,13 @@ inline void count_launch(long long n = 1) { g_kernel_launches.fetch_add(n, std::
 
 // Host-side launchers (pm_kernels.cu / phi_kernels.cu).
 cudaError_t launch_build_texture(const uint8_t* img, int W, int H, uint2* tex, cudaStream_t s);   // pitch tex_pitch(W)
-cudaError_t launch_init(const RefConst& rc, float* view_cost, cudaStream_t s);
+cudaError_t launch_init(const RefConst& rc, cudaStream_t s);
 cudaError_t launch_cost(const RefConst& rc, const float4* plane, float* cost, float* view_cost, cudaStream_t s);
-cudaError_t launch_phase(const RefConst& rc, int phase, cudaStream_t s);
+// one checkerboard phase (first: the first of the call, whose perturbations are drawn in any case)
+cudaError_t launch_phase(const RefConst& rc, int phase, bool first, cudaStream_t s);
+// bytes of the stored window of one pixel, and their construction into rc.win
+size_t pm_window_bytes(const RefConst& rc);
+cudaError_t launch_windows(const RefConst& rc, cudaStream_t s);
 // clears the candidate memo of rc's view (before the first phase of a call)
 cudaError_t launch_memo_reset(const RefConst& rc, cudaStream_t s);
 cudaError_t prime_launch_configs(const RefConst& rc);

@@ -81,6 +81,23 @@ __device__ __forceinline__ float gsum(float v) {
     return v;
 }
 
+// Sums of three values over each group of G lanes, in the same tree as gsum
+// but with the lanes sharing the work after the first step (6 shuffles for
+// G = 16 instead of 12): lane 0 of the group ends with a's sum, lane G / 2
+// with b's and lane G / 4 with c's.
+template <int G>
+__device__ __forceinline__ float gsum3(float a, float b, float c) {
+    const bool h = threadIdx.x & (G / 2), q = threadIdx.x & (G / 4);
+    float v = h ? b : a;
+    v += __shfl_xor_sync(0xffffffffu, h ? a : b, G / 2);
+    c += __shfl_xor_sync(0xffffffffu, c, G / 2);
+    float w = q ? c : v;
+    w += __shfl_xor_sync(0xffffffffu, q ? v : c, G / 4);
+#pragma unroll
+    for (int o = G / 8; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    return w;
+}
+
 template <int G>
 __device__ __forceinline__ unsigned group_mask(int lane) {
     return G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
@@ -171,14 +188,59 @@ struct __align__(16) WinGeo {
 // warp holds the same pixel's window (sample k = slot * G + lane_in_group).
 template <int S>
 struct PixWin {
-    __half2 o2[S];        // sample offsets / step: (k_u - r_now, k_v - r_now), exact in fp16 (the first
-                          // included sample for padding / excluded samples)
+    uint32_t o2[S];       // sample offsets / step: (k_u - r_now, k_v - r_now) as two bf16, exact (pack_offset; the
+                          // first included sample for padding / excluded samples)
     float w[S];           // bilateral weights (0 for padding / excluded)
     float wr[S];          // w * (I_ref - weighted mean)
     float mean;           // weighted mean of the reference samples
     WinGeo geo;
     bool ok;              // pixel exists and its reference patch is not flat
 };
+
+// Two offsets of at most 10.5 in steps of 1/2 as bf16 (exact: at most five
+// significant bits), x in the low half.  A bf16 widens with a shift or a mask
+// (integer pipe), an fp16 with a conversion on the multiply-add pipe, which
+// the sample loop keeps busier.
+__device__ __forceinline__ uint32_t pack_offset(float x, float y) {
+    return (__float_as_uint(x) >> 16) | (__float_as_uint(y) & 0xffff0000u);
+}
+__device__ __forceinline__ float2 unpack_offset(uint32_t o) {
+    return make_float2(__uint_as_float(o << 16), __uint_as_float(o & 0xffff0000u));
+}
+
+// window rows / columns inside the reference image: lane k tests offset k
+// (n <= 22 < 32)
+__device__ __forceinline__ void window_range(const RefConst& rc, int px, int py, int& ku_lo, int& ku_hi, int& kv_lo,
+                                             int& kv_hi) {
+    const int lane = threadIdx.x & 31, n = rc.n;
+    const float half = 0.5f * (float)(n - 1);
+    const float o = rc.step * ((float)lane - half);
+    const float eu = (float)px + o, ev = (float)py + o;
+    const unsigned mu = __ballot_sync(0xffffffffu, lane < n && eu >= 0.0f && eu <= (float)(rc.W - 1));
+    const unsigned mv = __ballot_sync(0xffffffffu, lane < n && ev >= 0.0f && ev <= (float)(rc.H - 1));
+    ku_lo = mu ? __ffs(mu) - 1 : n;
+    ku_hi = mu ? 31 - __clz(mu) : -1;
+    kv_lo = mv ? __ffs(mv) - 1 : n;
+    kv_hi = mv ? 31 - __clz(mv) : -1;
+}
+
+// Sample offsets of a pixel whose window covers rows / columns [lo, hi];
+// excluded and padding samples sit on the first included sample (weight 0).
+template <int G, int S>
+__device__ __forceinline__ void window_offsets(const RefConst& rc, int ku_lo, int ku_hi, int kv_lo, int kv_hi,
+                                               uint32_t (&o2)[S]) {
+    const int lg = threadIdx.x & (G - 1), n = rc.n;
+    const float half = 0.5f * (float)(n - 1);
+    const uint32_t o2_pad = pack_offset((float)ku_lo - half, (float)kv_lo - half);
+    const float inv_n = rcp_approx((float)n);   // (k + 1/2) / n stays 1/(2n) away from integers
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        const int k = s * G + lg;
+        const int kv = (int)(((float)k + 0.5f) * inv_n), ku = k - kv * n;   // exact for k < 2^20
+        const bool in = k < n * n && ku >= ku_lo && ku <= ku_hi && kv >= kv_lo && kv <= kv_hi;
+        o2[s] = in ? pack_offset((float)ku - half, (float)kv - half) : o2_pad;
+    }
+}
 
 // Window offsets s*(k - r_now) (Sec. III-C); samples outside the reference
 // image are left out of the window.
@@ -187,21 +249,10 @@ __device__ __forceinline__ void build_window(const RefConst& rc, int px, int py,
     const int lane = threadIdx.x & 31, lg = lane & (G - 1);
     const int n = rc.n;
     const float half = 0.5f * (float)(n - 1);
-    // window rows / columns inside the reference image: lane k tests offset k
-    // (n <= 22 < 32)
     int ku_lo, ku_hi, kv_lo, kv_hi;
-    {
-        const float o = rc.step * ((float)lane - half);
-        const float eu = (float)px + o, ev = (float)py + o;
-        const unsigned mu = __ballot_sync(0xffffffffu, lane < n && eu >= 0.0f && eu <= (float)(rc.W - 1));
-        const unsigned mv = __ballot_sync(0xffffffffu, lane < n && ev >= 0.0f && ev <= (float)(rc.H - 1));
-        ku_lo = mu ? __ffs(mu) - 1 : n;
-        ku_hi = mu ? 31 - __clz(mu) : -1;
-        kv_lo = mv ? __ffs(mv) - 1 : n;
-        kv_hi = mv ? 31 - __clz(mv) : -1;
-    }
+    window_range(rc, px, py, ku_lo, ku_hi, kv_lo, kv_hi);
     // excluded and padding samples sit on the first included sample (weight 0)
-    const __half2 o2_pad = __floats2half2_rn((float)ku_lo - half, (float)kv_lo - half);
+    const uint32_t o2_pad = pack_offset((float)ku_lo - half, (float)kv_lo - half);
     const float rcen = exists ? 4.0f * (float)__ldg(rc.img + (long long)py * rc.W + px) : 0.0f;
     const float inv_n = rcp_approx((float)n);   // (k + 1/2) / n stays 1/(2n) away from integers
     float sw = 0.0f, swr = 0.0f;
@@ -219,7 +270,7 @@ __device__ __forceinline__ void build_window(const RefConst& rc, int px, int py,
             float dc = r - rcen;
             w = __expf(fmaf(rc.sp_coef, ou * ou + ov * ov, rc.col_coef * dc * dc));
         }
-        pw.o2[s] = in ? __floats2half2_rn(ku_f, kv_f) : o2_pad;
+        pw.o2[s] = in ? pack_offset(ku_f, kv_f) : o2_pad;
         pw.w[s] = w;
         pw.wr[s] = r;   // temporarily the intensity
         sw += w;
@@ -233,9 +284,9 @@ __device__ __forceinline__ void build_window(const RefConst& rc, int px, int py,
 #pragma unroll
     for (int s = 0; s < S; ++s) {
         float d = pw.wr[s] - mu;
-        float t = pw.w[s] * d;
+        float t = __fmul_rn(pw.w[s], d);
         pw.wr[s] = t;
-        wrs += t;
+        wrs = __fadd_rn(wrs, t);   // not contracted: every kernel builds the same window
         srr = fmaf(t, d, srr);
     }
     srr = gsum<G>(srr);
@@ -258,6 +309,54 @@ __device__ __forceinline__ void build_window(const RefConst& rc, int px, int py,
     g.rlen = sqrtf(g.rx0 * g.rx0 + g.rx1 * g.rx1 + g.rx2 * g.rx2);
 }
 
+// Stored windows.  The reference side of a pixel's window does not depend on
+// the plane, so a call that visits each pixel several times builds it once
+// (k_init, k_window) and the phases read it back: per pixel a record of
+// S x G (w, wr) pairs in sample order, then WinGeo, then the usable flag.
+constexpr int kWinTail = 16;   // floats after the pairs: WinGeo (12), flag, padding
+__host__ __device__ constexpr int win_record_floats(int G, int S) { return 2 * G * S + kWinTail; }
+
+template <int G, int S>
+__device__ __forceinline__ void store_window(float* rec, const PixWin<S>& pw) {
+    constexpr int NG = 32 / G;
+    const int lane = threadIdx.x & 31, lg = lane & (G - 1), grp = lane / G;
+    if (pw.ok) {
+        // every group holds the same window: group g stores the slots g, g + NG, ...
+#pragma unroll
+        for (int s0 = 0; s0 < S; s0 += NG) {
+            float2 v = make_float2(pw.w[s0], pw.wr[s0]);
+#pragma unroll
+            for (int q = 1; q < NG; ++q)
+                if (s0 + q < S && grp == q) v = make_float2(pw.w[s0 + q], pw.wr[s0 + q]);
+            if (s0 + grp < S) __stcs(reinterpret_cast<float2*>(rec) + (s0 + grp) * G + lg, v);
+        }
+    }
+    if (lane == 0) {
+        float4* t = reinterpret_cast<float4*>(rec + 2 * G * S);
+        const WinGeo& g = pw.geo;
+        __stcs(t, make_float4(g.cu_lo, g.cu_hi, g.cv_lo, g.cv_hi));
+        __stcs(t + 1, make_float4(g.rx0, g.rx1, g.rx2, g.rlen));
+        __stcs(t + 2, make_float4(g.inv_wsum, g.srr, g.wr_sum, g.wsum));
+        __stcs(t + 3, make_float4(pw.ok ? 1.0f : 0.0f, 0.0f, 0.0f, 0.0f));
+    }
+}
+
+// Copies a record into the warp's shared memory in the background (16-byte
+// asynchronous copies through L2, off the L1 that the gathers live in).
+template <int G, int S>
+__device__ __forceinline__ void fetch_window(float* dst, const float* rec) {
+    constexpr int W16 = win_record_floats(G, S) / 4;
+    const int lane = threadIdx.x & 31;
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+#pragma unroll
+    for (int i = 0; i < W16; i += 32)
+        if (i + lane < W16)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16u * (uint32_t)(i + lane)),
+                         "l"(rec + 4 * (i + lane))
+                         : "memory");
+}
+__device__ __forceinline__ void fetch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Source-view constants copied to shared memory once per block (128 bytes,
 // read as 16-byte words, and 16 bytes of padding: lanes that read different
 // views' records at the same offset then fall on different banks): the
@@ -266,9 +365,8 @@ __device__ __forceinline__ void build_window(const RefConst& rc, int px, int py,
 struct __align__(16) ViewSm {
     const uint2* tex;
     uint32_t pitch;
-    float fold_x;         // 2 + 2 alpha: the guard texel and tex_fold's alpha in doubled coordinates
     uint32_t last;        // last texel index pitch (H + 1) - 1
-    float fold_y;         // 2 + 2 beta
+    float fold_x, fold_y; // 2 + 2 alpha, 2 + 2 beta: the guard texel and tex_fold in doubled coordinates
     float xmax2, ymax2;   // 2 W - 3, 2 H - 3: doubled, half-shifted image bounds
     float gx0, gx1, gy0, gy1;   // G_0, G_1 columns 0 and 1 (hi)
     float gz0, gz1, bxh, byh;   // G_2 columns 0 and 1 (hi); B_0, B_1 (hi)
@@ -279,8 +377,8 @@ struct __align__(16) ViewSm {
     float pad_[4];
 };
 
-static_assert(sizeof(ViewSm) == 144 && offsetof(ViewSm, pitch) == 8 && offsetof(ViewSm, fold_x) == 12 &&
-                  offsetof(ViewSm, last) == 16 && offsetof(ViewSm, fold_y) == 20 && offsetof(ViewSm, xmax2) == 24 &&
+static_assert(sizeof(ViewSm) == 144 && offsetof(ViewSm, pitch) == 8 && offsetof(ViewSm, last) == 12 &&
+                  offsetof(ViewSm, fold_x) == 16 && offsetof(ViewSm, fold_y) == 20 && offsetof(ViewSm, xmax2) == 24 &&
                   offsetof(ViewSm, gx0) == 32 &&
                   offsetof(ViewSm, gz0) == 48 && offsetof(ViewSm, bzh) == 64 && offsetof(ViewSm, gx2) == 80 &&
                   offsetof(ViewSm, gx0l) == 96 && offsetof(ViewSm, gy1l) == 112,
@@ -384,7 +482,8 @@ __device__ __forceinline__ Cand make_cand(const RefConst& rc, const PixWin<S>& p
 // per sample step, s j0 and s j1 (and s h0z, s h1z), so that a sample at
 // (k_u - r_now, k_v - r_now) steps from the pixel multiplies them by its
 // step counts directly; it also holds the magic numbers 1.5 * 2^24 +
-// (ax, ay) of tex_sample and (hypothesis | view << 8).
+// (ax, ay) of tex_sample and (hypothesis | view << 8 | fp16 coefficient a of
+// the texel at the anchor << 16).
 struct __align__(16) PairSm {
     float j0x, j0y, h0z, j1x;
     float j1y, h1z, nx, ny;
@@ -444,22 +543,15 @@ struct PairGeo {
 // enters through the fp16 coefficient a in one mixed add): the bilateral
 // weights favour samples like the centre, so the weighted mean lies near c0
 // and the one-pass moments rarely cancel.
-//   CENTRED = false: nc0 = -c0 out; sa, sb, se += sum w d, sum w d^2,
-//     sum w r' d over the lane's samples, d = s - c0;
-//   CENTRED = true: nc0 in (from the first pass, so every d is the same
-//     float); sa += sum w (d - mean_d)^2.
-// The gathers run in chunks of up to 8 slots (registers).
-template <int G, int S, bool CENTRED, int CH = (S <= 9 ? S : 8)>
+//   CENTRED = false: sa, sb, se += sum w d, sum w d^2, sum w r' d over the
+//     lane's samples, d = s - c0 (nc0 = -c0);
+//   CENTRED = true: sa += sum w (d - mean_d)^2.
+// The gathers run in chunks of up to 9 slots (registers).
+template <int G, int S, bool CENTRED, int CH = (S <= 9 ? S : (S + 1) / 2)>
 __device__ __forceinline__ void window_pass(const PixWin<S>& pw, int grp,
                                             const uint2* __restrict__ tex, uint32_t pitch, uint32_t last,
-                                            const PairGeo& g, float& nc0, float mean_d, float& sa, float& sb,
+                                            const PairGeo& g, float nc0, float mean_d, float& sa, float& sb,
                                             float& se) {
-    if (!CENTRED) {
-        // the texel at the anchor: X / Z = 0 in the sample formula below
-        const uint32_t ia = (uint32_t)__float_as_int(g.my) * pitch + (uint32_t)__float_as_int(g.mx);
-        const uint2 qa = __ldg(tex + min(ia, last));
-        nc0 = -__half2float(__ushort_as_half((unsigned short)(qa.x & 0xffffu)));
-    }
 #pragma unroll
     for (int k0 = 0; k0 < S; k0 += CH) {
         uint2 tq[CH];
@@ -468,7 +560,7 @@ __device__ __forceinline__ void window_pass(const PixWin<S>& pw, int grp,
         for (int kk = 0; kk < CH; ++kk) {
             const int k = k0 + kk;
             if (k < S) {
-                const float2 o = __half22float2(pw.o2[k]);
+                const float2 o = unpack_offset(pw.o2[k]);
                 const float X = fmaf(o.x, g.j0x, fmaf(o.y, g.j1x, g.nx));
                 const float Y = fmaf(o.x, g.j0y, fmaf(o.y, g.j1y, g.ny));
                 const float Z = fmaf(o.x, g.h0z, fmaf(o.y, g.h1z, g.pz));
@@ -495,8 +587,8 @@ __device__ __forceinline__ void window_pass(const PixWin<S>& pw, int grp,
                     sa = fmaf(pw.w[k] * e, e, sa);
                 } else {
                     // first and second moments in one pass
-                    const float t = pw.w[k] * dv;
-                    sa += t;
+                    const float t = __fmul_rn(pw.w[k], dv);
+                    sa = __fadd_rn(sa, t);
                     sb = fmaf(t, dv, sb);
                     se = fmaf(pw.wr[k], dv, se);
                 }
@@ -511,20 +603,15 @@ __device__ __forceinline__ void window_pass(const PixWin<S>& pw, int grp,
 // accumulated in FP32.  The coefficient a is shifted by c0 in fp16 (both
 // are integers up to 1020, so a - c0 is exact); c0 is the anchor texel's a,
 // as in window_pass.
-//   MODE 0: nc0 = -c0 out; sa, sb, se += sum w d, sum w d^2, sum w r' d;
+//   MODE 0: sa, sb, se += sum w d, sum w d^2, sum w r' d (nc0 = -c0);
 //   MODE 1: sa += sum w (d - mean_d)^2 in FP32;
 //   MODE 2: sd += the same in FP64 (the variance denominator near the
 //           flat-patch limit).
 // d is the same value in every mode (the same half2 operations).
-template <int G, int S, int MODE, int CH = (S <= 9 ? S : 8)>
+template <int G, int S, int MODE, int CH = (S <= 9 ? S : (S + 1) / 2)>
 __device__ __forceinline__ void window_pass_h2(const PixWin<S>& pw, const uint2* __restrict__ tex, uint32_t pitch,
-                                               uint32_t last, const PairGeo& g, float& nc0, float mean_d, float& sa,
+                                               uint32_t last, const PairGeo& g, float nc0, float mean_d, float& sa,
                                                float& sb, float& se, double& sd) {
-    const uint32_t ia = (uint32_t)__float_as_int(g.my) * pitch + (uint32_t)__float_as_int(g.mx);
-    if (MODE == 0) {
-        const uint2 qa = __ldg(tex + min(ia, last));
-        nc0 = -__half2float(__ushort_as_half((unsigned short)(qa.x & 0xffffu)));
-    }
     const __half2 c2 = __float2half2_rn(-nc0);   // exact: an integer <= 1020
 #pragma unroll
     for (int k0 = 0; k0 < S; k0 += CH) {
@@ -534,7 +621,7 @@ __device__ __forceinline__ void window_pass_h2(const PixWin<S>& pw, const uint2*
         for (int kk = 0; kk < CH; ++kk) {
             const int k = k0 + kk;
             if (k < S) {
-                const float2 o = __half22float2(pw.o2[k]);
+                const float2 o = unpack_offset(pw.o2[k]);
                 const float X = fmaf(o.x, g.j0x, fmaf(o.y, g.j1x, g.nx));
                 const float Y = fmaf(o.x, g.j0y, fmaf(o.y, g.j1y, g.ny));
                 const float Z = fmaf(o.x, g.h0z, fmaf(o.y, g.h1z, g.pz));
@@ -550,7 +637,7 @@ __device__ __forceinline__ void window_pass_h2(const PixWin<S>& pw, const uint2*
         for (int kk = 0; kk < CH; kk += 2) {
             const int k = k0 + kk;
             if (k < S) {
-                const bool two = k + 1 < S;   // compile-time
+                const bool two = kk + 1 < CH && k + 1 < S;   // compile-time
                 const uint2 q0 = tq[kk], q1 = two ? tq[kk + 1] : tq[kk];
                 uint32_t ab = __byte_perm(q0.x, q1.x, 0x5410), bb = __byte_perm(q0.x, q1.x, 0x7632);
                 uint32_t cb = __byte_perm(q0.y, q1.y, 0x5410), db = __byte_perm(q0.y, q1.y, 0x7632);
@@ -566,8 +653,8 @@ __device__ __forceinline__ void window_pass_h2(const PixWin<S>& pw, const uint2*
                     const float d = h ? dv.y : dv.x;
                     const float w = pw.w[k + h];
                     if (MODE == 0) {
-                        const float t = w * d;
-                        sa += t;
+                        const float t = __fmul_rn(w, d);
+                        sa = __fadd_rn(sa, t);
                         sb = fmaf(t, d, sb);
                         se = fmaf(pw.wr[k + h], d, se);
                     } else if (MODE == 1) {
@@ -690,8 +777,14 @@ __device__ __forceinline__ float eval_batch(const RefConst& rc, const ViewSm* __
             qw[1] = make_float4(j1y * st, h1z * st, nx, ny);
             // magic numbers with the anchor, the texture's guard texel and the
             // index fold (tex_fold): bits(ty) pitch + bits(tx) = texel index
-            const float fx = reinterpret_cast<const float4*>(sv + j)[0].w;
-            qw[2] = make_float4(pz, kMagic2 + (ax + fx), kMagic2 + (ay + w1.y), __int_as_float(c | (j << 8)));
+            const float mx = kMagic2 + (ax + w1.x), my = kMagic2 + (ay + w1.y);
+            // coefficient a of the texel at the anchor (X / Z = 0 in the sample
+            // formula), read here by one lane per pair
+            const uint4 v0 = reinterpret_cast<const uint4*>(sv + j)[0];
+            const uint2* tex = reinterpret_cast<const uint2*>(((unsigned long long)v0.y << 32) | v0.x);
+            const uint32_t ia = (uint32_t)__float_as_int(my) * v0.z + (uint32_t)__float_as_int(mx);
+            const uint32_t a16 = __ldg(reinterpret_cast<const unsigned short*>(tex + min(ia, v0.w)));
+            qw[2] = make_float4(pz, mx, my, __uint_as_float((uint32_t)c | ((uint32_t)j << 8) | (a16 << 16)));
         } else if (act) {
             tab[c * V + j] = 0.0f;   // view excluded for this hypothesis
         }
@@ -708,82 +801,69 @@ __device__ __forceinline__ float eval_batch(const RefConst& rc, const ViewSm* __
         float4* qw = reinterpret_cast<float4*>(pairs + (has ? it : 0));
         const float4 qa = qw[0], qb = qw[1], qc = qw[2];
         const PairGeo pg{qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w, qc.x, qc.y, qc.z};
-        const int cj = __float_as_int(qc.w), pj = cj >> 8;
-        // view words 0 (texels, pitch) and 1 (last texel)
-        const uint4 v0 = reinterpret_cast<const uint4*>(sv + pj)[0];
-        const uint32_t v_last = reinterpret_cast<const uint4*>(sv + pj)[1].x;
+        const uint32_t cj = __float_as_uint(qc.w);
+        const float nc0 = -__half2float(__ushort_as_half((unsigned short)(cj >> 16)));
+        // view word 0: texels, pitch, last texel
+        const uint4 v0 = reinterpret_cast<const uint4*>(sv + ((cj >> 8) & 31u))[0];
         const uint2* v_tex = reinterpret_cast<const uint2*>(((unsigned long long)v0.y << 32) | v0.x);
-        float sa = 0.0f, sb = 0.0f, se = 0.0f, sdd, mean_d;
+        float sa = 0.0f, sb = 0.0f, se = 0.0f;
         if constexpr (!MIXED) {
-            float nc0 = 0.0f;
-            window_pass<G, S, false>(pw, grp, v_tex, v0.z, v_last, pg, nc0, 0.0f, sa, sb, se);
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) {
-                sa += __shfl_xor_sync(0xffffffffu, sa, o);
-                sb += __shfl_xor_sync(0xffffffffu, sb, o);
-                se += __shfl_xor_sync(0xffffffffu, se, o);
-            }
-            mean_d = sa * inv_wsum;
-            // sum w (s - mu)^2 = sum w d^2 - mu_d sum w d (one pass)
-            sdd = fmaf(-mean_d, sa, sb);
-            // when the shift lies far from the patch mean, W mu_d^2 > 8 sum
-            // w (d - mu_d)^2, the one-pass form loses bits to cancellation:
-            // the samples are taken again for the centred second moment (the
-            // two-pass form of Eq. 4)
-            const bool centre = has && sa * mean_d > 8.0f * sdd;
-            if (__any_sync(0xffffffffu, centre)) {
-                float s2 = 0.0f, u0 = 0.0f, u1 = 0.0f;
-                window_pass<G, S, true>(pw, grp, v_tex, v0.z, v_last, pg, nc0, mean_d, s2, u0,
-                                                u1);
-                s2 = gsum<G>(s2);
-                if (centre) sdd = s2;
-            }
+            window_pass<G, S, false>(pw, grp, v_tex, v0.z, v0.w, pg, nc0, 0.0f, sa, sb, se);
         } else {
-            float nc0 = 0.0f;
-            {
+            double unused = 0.0;
+            window_pass_h2<G, S, 0>(pw, v_tex, v0.z, v0.w, pg, nc0, 0.0f, sa, sb, se, unused);
+        }
+        // lane 0 of the group: sa, and sb from lane G / 2; lane G / 4: se
+        const float tot = gsum3<G>(sa, sb, se);
+        const float sb0 = __shfl_xor_sync(0xffffffffu, tot, G / 2);
+        const bool first = has && lg == 0;
+        float mean_d = tot * inv_wsum;
+        // sum w (s - mu)^2 = sum w d^2 - mu_d sum w d (one pass)
+        float sdd = fmaf(-mean_d, tot, sb0);
+        // when the shift lies far from the patch mean, W mu_d^2 > 8 sum
+        // w (d - mu_d)^2, the one-pass form loses bits to cancellation:
+        // the samples are taken again for the centred second moment (the
+        // two-pass form of Eq. 4)
+        const bool centre = first && tot * mean_d > 8.0f * sdd;
+        if (__any_sync(0xffffffffu, centre)) {
+            const float md = __shfl_sync(0xffffffffu, mean_d, lane & ~(G - 1));
+            float s2 = 0.0f, u0 = 0.0f, u1 = 0.0f;
+            if constexpr (!MIXED) {
+                window_pass<G, S, true>(pw, grp, v_tex, v0.z, v0.w, pg, nc0, md, s2, u0, u1);
+            } else {
                 double unused = 0.0;
-                window_pass_h2<G, S, 0>(pw, v_tex, v0.z, v_last, pg, nc0, 0.0f, sa, sb, se, unused);
+                window_pass_h2<G, S, 1>(pw, v_tex, v0.z, v0.w, pg, nc0, md, s2, u0, u1, unused);
             }
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) {
-                sa += __shfl_xor_sync(0xffffffffu, sa, o);
-                sb += __shfl_xor_sync(0xffffffffu, sb, o);
-                se += __shfl_xor_sync(0xffffffffu, se, o);
-            }
-            mean_d = sa * inv_wsum;
-            sdd = fmaf(-mean_d, sa, sb);
-            // the shift far from the patch mean: the centred second moment in
-            // FP32 from a second gather pass, as in the FP32 path
-            const bool centre = has && sa * mean_d > 8.0f * sdd;
-            if (__any_sync(0xffffffffu, centre)) {
-                float s2 = 0.0f, u0 = 0.0f, u1 = 0.0f;
-                double unused = 0.0;
-                window_pass_h2<G, S, 1>(pw, v_tex, v0.z, v_last, pg, nc0, mean_d, s2, u0, u1, unused);
-                s2 = gsum<G>(s2);
-                if (centre) sdd = s2;
-            }
+            s2 = gsum<G>(s2);
+            if (centre) sdd = s2;
+        }
+        if constexpr (MIXED) {
             // a source patch within 1 % of the flat limit (where the exclusion
             // decision is taken): the variance denominator in FP64
-            const bool near_flat = has && sdd < 1.01f * kTauVar * geo.wsum && sdd > 0.99f * kTauVar * geo.wsum;
+            const bool near_flat =
+                first && sdd < 1.01f * kTauVar * geo.wsum && sdd > 0.99f * kTauVar * geo.wsum;
             if (__any_sync(0xffffffffu, near_flat)) {
+                const float md = __shfl_sync(0xffffffffu, mean_d, lane & ~(G - 1));
                 double v = 0.0;
                 float s0 = 0.0f, u0 = 0.0f, u1 = 0.0f;
-                window_pass_h2<G, S, 2, 2>(pw, v_tex, v0.z, v_last, pg, nc0, mean_d, s0, u0, u1, v);
+                window_pass_h2<G, S, 2, 2>(pw, v_tex, v0.z, v0.w, pg, nc0, md, s0, u0, u1, v);
 #pragma unroll
                 for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                 if (near_flat) sdd = (float)v;
             }
         }
-        if (has && lg == 0) qw[0] = make_float4(sdd, se, mean_d, __int_as_float(cj));
+        // over the record's first word, which is not read again
+        if (first) *reinterpret_cast<float2*>(qw) = make_float2(sdd, mean_d);
+        if (has && lg == G / 4) reinterpret_cast<float*>(qw)[2] = tot;
     }
     __syncwarp();
     // ---- 2b. per evaluated pair, one per lane: ZNCC (Eq. 4), C(x, j) = 1 - Z
     // and its Eq. 5 weight
     for (int i = lane; i < count; i += 32) {
         const float4 q = reinterpret_cast<const float4*>(pairs + i)[0];
-        const int cj = __float_as_int(q.w), pj = cj >> 8, pc = cj & 255;
+        const int cj = pairs[i].cj, pj = (cj >> 8) & 31, pc = cj & 255;
         // sum w r' (s - mu) = sum w r' d - mu_d sum w r'
-        const float srd = fmaf(-q.z, geo.wr_sum, q.y);
+        const float srd = fmaf(-q.y, geo.wr_sum, q.z);
         const bool flat = !(q.x >= kTauVar * geo.wsum);
         const float z = fminf(1.0f, fmaxf(-1.0f, srd * rsqrtf(geo.srr * q.x)));
         const float cjv = flat ? kCmax : fminf(1.0f - z, kCmax);
@@ -796,6 +876,7 @@ __device__ __forceinline__ float eval_batch(const RefConst& rc, const ViewSm* __
     int cnt = 0;
     float inv_sum = 0.0f;
     if ((okm >> lane) & 1u)
+#pragma unroll 4
         for (int j = 0; j < V; ++j) {
             const float wv = tab[lane * V + j];
             cnt += wv > 0.0f;
@@ -829,22 +910,6 @@ __device__ __forceinline__ int warp_argmin(float cost, int nc, float& best) {
     }
     best = c;
     return i;
-}
-
-// Sec. III-B: n = (cos t sin p, sin t sin p, cos p), turned to face the camera.
-__device__ __forceinline__ void normal_from_angles(float th, float ph, float rx0, float rx1, float rx2, float& n0,
-                                                   float& n1, float& n2) {
-    float st, ct, sp, cp;
-    sincosf(th, &st, &ct);
-    sincosf(ph, &sp, &cp);
-    n0 = ct * sp;
-    n1 = st * sp;
-    n2 = cp;
-    if (n0 * rx0 + n1 * rx1 + n2 * rx2 > 0.0f) {
-        n0 = -n0;
-        n1 = -n1;
-        n2 = -n2;
-    }
 }
 
 }  // namespace mvsdev

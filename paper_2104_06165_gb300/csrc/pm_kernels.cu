@@ -40,72 +40,75 @@ __global__ void k_build_texture(const uint8_t* __restrict__ img, int W, int H, i
 
 // Per-block shared memory: the source-view table and one pair list per warp.
 constexpr int kWarps = kBlock / 32;
-// Checkerboard-phase blocks cover a tile of kTileX x kTileY pixels of the
-// active colour, one warp per pixel, so that the warps sharing an SM's L1
-// gather overlapping windows.  20 warps at 96 registers a thread hide more
-// gather latency than 16 at 128 (4 % less time per phase at 3072 x 2048
-// with 11 x 11 samples; 12, 21 and 24 warps were slower), and a tall tile
-// of 2 x 10 warps (4 x 10 pixels) shares more of the L1 than 4 x 5 (4 %
-// less again; 10 x 2 and 5 x 4 were slower, 1 x 20 the same).
-#ifndef MVS_TILE_X
-#define MVS_TILE_X 2
-#endif
-#ifndef MVS_TILE_Y
-#define MVS_TILE_Y 10
-#endif
-// Windows of 16 slots per lane need more than 128 registers: their blocks
-// keep to one row of kTileX pixels (12 warps per SM).
+// Checkerboard phases: one block per SM whose warps take single pixels of the
+// active colour from the block's tiles, 1 x kTileY such pixels each.  A short
+// tile leaves the blocks even (320 x 240, 3 iterations: 1108 us with 8 pixels,
+// 1139 with 16, 1239 with 32; 1511 x 1007 the same within 1 %), a vertical
+// one shares more L1 lines than a square (2 x 10: 4 % slower).
+constexpr int kTileY = 8;
+// Warps of the block: with the windows read back, 24 warps at 80 registers (a
+// few spilled outside the sample loop) hide more latency than 20 at 96 (1511 x
+// 1007, 8 iterations: 75.0 against 78.2 ms; 16 warps 78.6, 28 warps 75.5).
+// Layouts with more slots per lane need the registers.
 template <int S>
-struct PhaseTile {
-    static constexpr int TX = MVS_TILE_X;
-    static constexpr int TY = S >= 16 ? 1 : MVS_TILE_Y;
-    static constexpr int WARPS = TX * TY;
-    static constexpr int BLOCK = 32 * WARPS;
-    static constexpr int MIN_BLOCKS = (S >= 16 ? 384 : 512) / BLOCK > 0 ? (S >= 16 ? 384 : 512) / BLOCK : 1;
-};
+constexpr int phase_max_warps() { return S <= 9 ? 24 : S <= 11 ? 20 : S <= 14 ? 16 : 12; }
 
 // Blocks of the one-hypothesis kernels per SM: 5 (96 registers, no spills)
 // for windows of up to 9 slots per lane; 16 slots need more registers.
 template <int S>
-constexpr int one_hyp_blocks() { return S >= 16 ? 1 : 5; }
+constexpr int one_hyp_blocks() { return S <= 9 ? 5 : S <= 11 ? 4 : S <= 14 ? 3 : 1; }
 
 // ---------------------------------------------------------------------------
 // Sec. III-B: random initialisation, then the cost of the initial plane.
 // One warp per pixel, grid-stride over the pixels.
 // ---------------------------------------------------------------------------
 template <int G, int S, bool MIXED>
-__global__ void __launch_bounds__(kBlock, one_hyp_blocks<S>()) k_init(const __grid_constant__ RefConst rc, float* view_cost) {
+__global__ void __launch_bounds__(kBlock, one_hyp_blocks<S>()) k_init(const __grid_constant__ RefConst rc) {
     extern __shared__ __align__(16) unsigned char smem[];
     ViewSm* views = reinterpret_cast<ViewSm*>(smem);
     load_views(rc, views);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long npix = (long long)rc.W * rc.H;
-    unsigned nev = 0;
-    for (long long a = (long long)blockIdx.x * kWarps + warp; a < npix; a += (long long)gridDim.x * kWarps) {
+    unsigned nev = 0, it = 0;
+    // the draws of this warp's next 32 pixels, one per lane: the depth's
+    // uniform and the normal before it is turned to the camera
+    float u0 = 0.0f, dn0 = 0.0f, dn1 = 0.0f, dn2 = 0.0f;
+    for (long long a = (long long)blockIdx.x * kWarps + warp; a < npix; a += (long long)gridDim.x * kWarps, ++it) {
         const int px = (int)(a % rc.W), py = (int)(a / rc.W);
         PixWin<S> pw;
         build_window<G, S>(rc, px, py, true, pw);
-        float u[3];
-        draws3(rc, a, -1, u);
-        float d = rc.d_lo + (rc.d_hi - rc.d_lo) * u[0];
+        if (rc.win) store_window<G, S>(rc.win + a * win_record_floats(G, S), pw);
+        if ((it & 31u) == 0) {
+            float u[3];
+            draws3(rc, a + (long long)lane * gridDim.x * kWarps, -1, u);
+            float st, ct, sp, cp;
+            sincosf(2.0f * kPi * u[1], &st, &ct);
+            sincosf(kPi * (u[2] - 0.5f), &sp, &cp);
+            u0 = u[0];
+            dn0 = ct * sp;
+            dn1 = st * sp;
+            dn2 = cp;
+        }
+        const float u = __shfl_sync(0xffffffffu, u0, it & 31u);
+        float n0 = __shfl_sync(0xffffffffu, dn0, it & 31u), n1 = __shfl_sync(0xffffffffu, dn1, it & 31u);
+        float n2 = __shfl_sync(0xffffffffu, dn2, it & 31u);
+        float d = rc.d_lo + (rc.d_hi - rc.d_lo) * u;
         if (rc.init_range) {   // Sec. III-B: a depth between the nearest sparse features
             const float2 r = rc.init_range[a];
-            if (r.x == r.x) d = r.x + (r.y - r.x) * u[0];
+            if (r.x == r.x) d = r.x + (r.y - r.x) * u;
         }
-        float th = 2.0f * kPi * u[1];
-        float ph = kPi * (u[2] - 0.5f);
-        float n0, n1, n2;
-        normal_from_angles(th, ph, pw.geo.rx0, pw.geo.rx1, pw.geo.rx2, n0, n1, n2);
-        float* vc = view_cost ? view_cost + a * rc.n_src : nullptr;
+        if (n0 * pw.geo.rx0 + n1 * pw.geo.rx1 + n2 * pw.geo.rx2 > 0.0f) {   // face the camera
+            n0 = -n0;
+            n1 = -n1;
+            n2 = -n2;
+        }
         float c = kCmax;
         if (pw.ok) {
             PixView* pv = warp_pixviews(smem, rc.n_src, warp);
             pix_views(rc, views, px, py, pv);
             Cand my = make_cand(rc, pw, pw.geo, n0, n1, n2, d, lane == 0);
-            c = eval_batch<G, S, true, MIXED>(rc, views, pw, pw.geo, pv, my, 1, warp_pairs(smem, rc.n_src, warp), vc,
-                                              nev);
-        } else if (vc && lane < rc.n_src) {
-            vc[lane] = kCmax;
+            c = eval_batch<G, S, false, MIXED>(rc, views, pw, pw.geo, pv, my, 1, warp_pairs(smem, rc.n_src, warp),
+                                               nullptr, nev);
         }
         if (lane == 0) {
             rc.plane[a] = make_float4(n0, n1, n2, d);
@@ -113,6 +116,18 @@ __global__ void __launch_bounds__(kBlock, one_hyp_blocks<S>()) k_init(const __gr
         }
     }
     flush_evals(rc.eval_counter, nev);
+}
+
+// the stored windows of a call that starts from given planes
+template <int G, int S>
+__global__ void __launch_bounds__(kBlock, one_hyp_blocks<S>()) k_window(const __grid_constant__ RefConst rc) {
+    const int warp = threadIdx.x >> 5;
+    const long long npix = (long long)rc.W * rc.H;
+    for (long long a = (long long)blockIdx.x * kWarps + warp; a < npix; a += (long long)gridDim.x * kWarps) {
+        PixWin<S> pw;
+        build_window<G, S>(rc, (int)(a % rc.W), (int)(a / rc.W), true, pw);
+        store_window<G, S>(rc.win + a * win_record_floats(G, S), pw);
+    }
 }
 
 // cost of a given plane map
@@ -175,65 +190,105 @@ __device__ __forceinline__ void group_member(int g, int k, int& dx, int& dy) {
     }
 }
 
+// The 8 groups x 16 member slots as the phase kernel scans them: entry
+// 16 g + k of the block's table is the pixel-index offset of member k of group
+// g and its (dx + 32) << 8 | (dy + 32), or -1 past the group's size.
+constexpr int kMemberSlots = 128, kReach = 25;   // members lie at most kReach pixels away
+__device__ __forceinline__ void fill_members(const RefConst& rc, int2* tab) {
+    for (int i = threadIdx.x; i < kMemberSlots; i += blockDim.x) {
+        const int g = i >> 4, k = i & 15;
+        int dx, dy;
+        group_member(g, k, dx, dy);
+        const bool in = k < (g < 4 ? 6 : 11);
+        tab[i] = in ? make_int2(dy * rc.W + dx, ((dx + 32) << 8) | (dy + 32)) : make_int2(0, -1);
+    }
+}
+
 // Member of group g with the lowest stored cost (in-image members only, the
-// first listed wins a tie), as a pixel index on lane g < 8, or -1.  The 8
-// groups x 16 member slots are spread over 4 registers of the warp (register
-// r, lane l: group 2r + l / 16, member l % 16), each half warp takes the
-// minimum of its register, and the lowest member holding it wins; stored
-// costs are >= 0, so their bit patterns order like the values.  The members
-// have the other colour, which this phase does not write.
-__device__ __forceinline__ int best_members(const RefConst& rc, int px, int py, int& member) {
-    const int lane = threadIdx.x & 31, half = lane >> 4, k = lane & 15;
+// first listed wins a tie), as a pixel index on lane g < 8, or -1, with its
+// position.  The 128 slots are spread over 4 registers of the warp (register
+// r, lane l: slot 32 r + l), each half warp takes the minimum of its register,
+// and the lowest member holding it wins; stored costs are >= 0, so their bit
+// patterns order like the values.  The members have the other colour, which
+// this phase does not write.  The table replaces the offset arithmetic and,
+// away from the image border, the bounds tests.
+__device__ __forceinline__ int best_members(const RefConst& rc, const int2* tab, int px, int py, int& member, int& x2,
+                                            int& y2) {
+    const int lane = threadIdx.x & 31, half = lane >> 4;
+    const int pix = py * rc.W + px;
+    const bool inner = px >= kReach && py >= kReach && px < rc.W - kReach && py < rc.H - kReach;   // warp-uniform
     unsigned first[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        const int g = 2 * r + half;
-        int dx, dy;
-        group_member(g, k, dx, dy);
-        const int x2 = px + dx, y2 = py + dy;
-        const bool in = k < (g < 4 ? 6 : 11) && x2 >= 0 && x2 < rc.W && y2 >= 0 && y2 < rc.H;
-        const unsigned bits = in ? __float_as_uint(__ldg(rc.cost + (long long)y2 * rc.W + x2) + 0.0f) : 0xffffffffu;
+        const int2 e = tab[32 * r + lane];
+        bool in = e.y >= 0;
+        if (!inner) {
+            const int x = px + (e.y >> 8) - 32, y = py + (e.y & 0xff) - 32;
+            in = in && x >= 0 && x < rc.W && y >= 0 && y < rc.H;
+        }
+        const unsigned bits = in ? __float_as_uint(__ldg(rc.cost + (pix + e.x)) + 0.0f) : 0xffffffffu;
         const unsigned mn0 = __reduce_min_sync(0xffffffffu, half ? 0xffffffffu : bits);
         const unsigned mn1 = __reduce_min_sync(0xffffffffu, half ? bits : 0xffffffffu);
         first[r] = __ballot_sync(0xffffffffu, in && bits == (half ? mn1 : mn0));
     }
     int q = -1;
     member = -1;
+    x2 = y2 = 0;
     if (lane < 8) {
-        const int g = lane;
-        const unsigned m = (first[g >> 1] >> (16 * (g & 1))) & 0xffffu;
+        const unsigned fm = lane & 4 ? (lane & 2 ? first[3] : first[2]) : (lane & 2 ? first[1] : first[0]);
+        const unsigned m = (fm >> (16 * (lane & 1))) & 0xffffu;
         if (m) {
-            int dx, dy;
             member = __ffs(m) - 1;
-            group_member(g, member, dx, dy);
-            q = (py + dy) * rc.W + px + dx;
+            const int2 e = tab[16 * lane + member];
+            x2 = px + (e.y >> 8) - 32;
+            y2 = py + (e.y & 0xff) - 32;
+            q = pix + e.x;
         }
     }
     return q;
 }
 
-// Refinement perturbations of one pixel, drawn ahead for the next 32 pixels
-// of a warp (one lane each): delta_d, and cos / sin of delta_theta and of
-// delta_phi.  20 bytes per pixel, after the pair lists; then each warp's
-// PhaseWarp record.
-// Per-warp state of the current pixel kept in shared memory rather than in
-// registers through the evaluation rounds: its window geometry, its plane and
-// cost so far, and the hypothesis each lane proposes in the current stage.
-struct __align__(16) PhaseWarp {
-    WinGeo geo;
-    float4 cur;
-    float cur_c, pad_[3];
-    float4 hyp[8];     // the stage's hypotheses (at most 8: propagation groups, proposals, refinement)
-};
-// Shared memory of a phase block (the same for both precisions).
-__host__ __device__ constexpr size_t phase_smem_bytes(int n_src, int warps, bool mixed) {
-    return (void)mixed,
-           smem_block_bytes(n_src, warps) + (size_t)warps * (32 * (sizeof(float4) + sizeof(float)) + sizeof(PhaseWarp));
+// Refinement perturbations (Sec. III-C) of one iteration, both colours, one
+// pixel per thread: delta_d in [-d_hi/4, d_hi/4], and cos / sin of
+// delta_theta in [-pi/2, pi/2] and of delta_phi in [-pi/12, pi/12].  Drawn
+// ahead of the phases: one pixel per lane, not one per warp.
+__global__ void __launch_bounds__(256) k_draws(const __grid_constant__ RefConst rc, int iter) {
+    const long long n = (long long)rc.W * rc.H;
+    for (long long a = blockIdx.x * 256LL + threadIdx.x; a < n; a += gridDim.x * 256LL) {
+        const int x = (int)(a % rc.W), y = (int)(a / rc.W);
+        float u[3];
+        draws3(rc, a, 2 * iter + ((x + y) & 1), u);
+        float sdt, cdt, sdp, cdp;
+        sincosf((2.0f * u[1] - 1.0f) * (kPi * 0.5f), &sdt, &cdt);
+        sincosf((2.0f * u[2] - 1.0f) * (kPi / 12.0f), &sdp, &cdp);
+        rc.draw4[a] = make_float4((2.0f * u[0] - 1.0f) * (rc.d_hi * 0.25f), cdt, sdt, cdp);
+        rc.draw1[a] = sdp;
+    }
 }
 
-// Rows of warps of a phase block: PhaseTile<S>::TY, or fewer when the
-// block's pair lists (which grow with the number of sources) would exceed the
-// per-block shared memory.
+// Per-warp state of the current pixel kept in shared memory rather than in
+// registers through the evaluation rounds: its window geometry, its plane and
+// cost so far, its perturbations, and the hypothesis each lane proposes in the
+// current stage.
+struct __align__(16) PhaseWarp {
+    WinGeo geo;
+    float draw[5];     // delta_d, cos / sin delta_theta, cos / sin delta_phi
+    float cur_c, pad_[2];
+    float4 cur;
+    float4 hyp[8];     // the stage's hypotheses (at most 8: propagation groups, proposals, refinement)
+};
+// Landing buffer of a warp (floats): the next pixel's perturbations (5, padded)
+// after its stored window (rec floats, 0 when windows are rebuilt).
+constexpr int kDrawFloats = 8;
+// Shared memory of a phase block (the same for both precisions).
+__host__ __device__ constexpr size_t phase_smem_bytes(int n_src, int warps, int rec) {
+    return smem_block_bytes(n_src, warps) +
+           (size_t)warps * (sizeof(PhaseWarp) + (size_t)(rec + kDrawFloats) * sizeof(float));
+}
+
+// Warps of a phase block: phase_max_warps<S>(), or fewer when the warps' pair
+// lists (which grow with the number of sources) would exceed the per-block
+// shared memory.
 // The limit is a property of the current device (queried once per device;
 // a failed query leaves 48 KB, the limit without the opt-in).
 int max_block_smem() {
@@ -249,83 +304,115 @@ int max_block_smem() {
     return v;
 }
 template <int S>
-int phase_rows(int n_src, bool mixed) {
-    int ty = PhaseTile<S>::TY;
-    while (ty > 1 && phase_smem_bytes(n_src, PhaseTile<S>::TX * ty, mixed) > (size_t)max_block_smem()) --ty;
-    return ty;
+int phase_warps(int n_src, int rec) {
+    int w = phase_max_warps<S>();
+    // the kernel's static shared memory (member table, queue) counts as well
+    while (w > 1 && phase_smem_bytes(n_src, w, rec) + kMemberSlots * sizeof(int2) + 64 > (size_t)max_block_smem()) --w;
+    return w;
 }
 
-// Tiles are visited in super-tiles of 8 x 16 tiles so that the pixels in
-// flight at once form a compact region (a smaller source footprint in L2;
-// within a phase the order of the pixels does not change the result).
-// Pixel of the active colour that warp `warp` takes in tile t, or -1.
-template <int TX>
-__device__ __forceinline__ long long phase_pixel(const RefConst& rc, long long t, int warp, int color, int TY,
-                                                 int& px, int& py) {
-    constexpr int kSTX = 8, kSTY = 16;
-    const int Wa = (rc.W + 1) >> 1;
-    const int ntx = (Wa + TX - 1) / TX, nty = (rc.H + TY - 1) / TY;
-    const int nstx = (ntx + kSTX - 1) / kSTX;
-    const int sti = (int)(t / (kSTX * kSTY)), r = (int)(t % (kSTX * kSTY));
-    const int tx = (sti % nstx) * kSTX + r % kSTX, ty = (sti / nstx) * kSTY + r / kSTX;
-    const int ax = tx * TX + warp % TX;
-    py = ty * TY + warp / TX;
-    px = 2 * ax + ((py + color) & 1);
-    if (tx >= ntx || ty >= nty || ax >= Wa || py >= rc.H || px >= rc.W) return -1;
-    return (long long)py * rc.W + px;
+// Tiles are visited in super-tiles of kSuperX x kSuperY tiles (fewer at the
+// right and lower edge) so that the pixels in flight at once form a compact
+// region (a smaller source footprint in L2; within a phase the order of the
+// pixels does not change the result).  Pixel of the active colour that slot
+// `slot` of tile t < ntx * nty covers, as y << 16 | x (sides are at most
+// 32768), or -1.
+constexpr int kSuperX = 8, kSuperY = 32;
+__device__ __forceinline__ int phase_pixel(const RefConst& rc, int t, int slot, int color, int ntx, int nty) {
+    const int sr = t / (kSuperY * ntx), r = t - sr * kSuperY * ntx;    // row of super-tiles
+    const int h = min(kSuperY, nty - kSuperY * sr);
+    const int sc = r / (kSuperX * h), r2 = r - sc * kSuperX * h;       // super-tile of the row
+    const int w = min(kSuperX, ntx - kSuperX * sc);
+    const int ry = r2 / w, rx = r2 - ry * w;
+    const int py = (sr * kSuperY + ry) * kTileY + slot, px = 2 * (sc * kSuperX + rx) + ((py + color) & 1);
+    return px < rc.W && py < rc.H ? (py << 16) | px : -1;
 }
 
-template <int G, int S, bool MIXED>
-__global__ void __launch_bounds__(PhaseTile<S>::BLOCK, PhaseTile<S>::MIN_BLOCKS)
+template <int G, int S, bool MIXED, bool STORED>
+__global__ void __launch_bounds__(32 * phase_max_warps<S>(), 1)
     k_phase(const __grid_constant__ RefConst rc, int phase) {
-    // the block is kTileX x kTileY warps, kTileY <= PhaseTile<S>::TY chosen by
-    // the host so that the block's shared memory fits
-    constexpr int kTileX = PhaseTile<S>::TX;
-    const int kTileY = (int)(blockDim.x >> 5) / kTileX;
-    const int kWarpsB = kTileX * kTileY;
-    extern __shared__ __align__(16) unsigned char smem[];   // phase_smem_bytes(n_src, kWarpsB, MIXED)
+    const int kWarpsB = (int)(blockDim.x >> 5);   // phase_warps<S>, chosen by the host
+    extern __shared__ __align__(16) unsigned char smem[];   // phase_smem_bytes(n_src, kWarpsB, record floats)
+    __shared__ int2 members[kMemberSlots];
+    __shared__ int queue;    // pixels of this block's tiles handed to its warps so far
     ViewSm* views = reinterpret_cast<ViewSm*>(smem);
-    load_views(rc, views);
+    fill_members(rc, members);
+    if (threadIdx.x == 0) queue = 0;
+    load_views(rc, views);   // (ends with a block barrier)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int color = phase & 1;
-    float4* draw4 = reinterpret_cast<float4*>(smem + smem_block_bytes(rc.n_src, kWarpsB)) + warp * 32;
-    float* draw1 = reinterpret_cast<float*>(reinterpret_cast<float4*>(smem + smem_block_bytes(rc.n_src, kWarpsB)) +
-                                            kWarpsB * 32) + warp * 32;
-    PhaseWarp* ws = reinterpret_cast<PhaseWarp*>(smem + smem_block_bytes(rc.n_src, kWarpsB) +
-                                                 (size_t)kWarpsB * 32 * (sizeof(float4) + sizeof(float))) + warp;
-    const int Wa = (rc.W + 1) >> 1;
-    const int ntx = (Wa + kTileX - 1) / kTileX, nty = (rc.H + kTileY - 1) / kTileY;
-    const int nstx = (ntx + 7) / 8, nsty = (nty + 15) / 16;
-    const long long ntiles = (long long)nstx * nsty * (8 * 16);
-    unsigned nev = 0, it = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
-        if ((it & 31u) == 0) {
-            // refinement perturbations (Sec. III-C) of this warp's next 32
-            // pixels, one per lane: delta_d in [-d_hi/4, d_hi/4],
-            // delta_theta in [-pi/2, pi/2], delta_phi in [-pi/12, pi/12]
-            int qx, qy;
-            const long long q = phase_pixel<kTileX>(rc, t + (long long)lane * gridDim.x, warp, color, kTileY, qx, qy);
-            float u[3];
-            draws3(rc, q < 0 ? 0 : q, phase, u);
-            float sdt, cdt, sdp, cdp;
-            sincosf((2.0f * u[1] - 1.0f) * (kPi * 0.5f), &sdt, &cdt);
-            sincosf((2.0f * u[2] - 1.0f) * (kPi / 12.0f), &sdp, &cdp);
-            __syncwarp();
-            draw4[lane] = make_float4((2.0f * u[0] - 1.0f) * (rc.d_hi * 0.25f), cdt, sdt, cdp);
-            draw1[lane] = sdp;
-            __syncwarp();
+    constexpr int kRec = STORED ? win_record_floats(G, S) : 0;
+    PhaseWarp* ws = reinterpret_cast<PhaseWarp*>(smem + smem_block_bytes(rc.n_src, kWarpsB)) + warp;
+    // the next pixel's stored window and perturbations land here while the
+    // current one is scored
+    float* land = reinterpret_cast<float*>(smem + smem_block_bytes(rc.n_src, kWarpsB) +
+                                           (size_t)kWarpsB * sizeof(PhaseWarp)) + (size_t)warp * (kRec + kDrawFloats);
+    const int ntx = (rc.W + 1) >> 1, nty = (rc.H + kTileY - 1) / kTileY;
+    // The block takes every gridDim.x-th tile and its warps draw the tiles'
+    // pixels from one queue, in order: the warps of an SM stay on neighbouring
+    // pixels (which share L1 lines) and end together, although the work of a
+    // pixel varies several-fold.  Returns a phase_pixel, or -1 at the end.
+    auto take = [&]() {
+        for (;;) {
+            int i = 0;
+            if (lane == 0) i = atomicAdd(&queue, 1);
+            i = __shfl_sync(0xffffffffu, i, 0);
+            const int t = (int)blockIdx.x + i / kTileY * (int)gridDim.x;
+            if (t >= ntx * nty) return -1;
+            const int p = phase_pixel(rc, t, i % kTileY, color, ntx, nty);
+            if (p >= 0) return p;
         }
-        int px, py;
-        const long long pix = phase_pixel<kTileX>(rc, t, warp, color, kTileY, px, py);
-        if (pix < 0) continue;   // warp-uniform
-        PixWin<S> pw;
-        build_window<G, S>(rc, px, py, true, pw);
-        if (!pw.ok) continue;                           // flat patch: every hypothesis costs C_max
-        // the window geometry and the pixel's state wait in shared memory
-        // (fewer live registers through the evaluation rounds)
+    };
+    auto fetch = [&](int p) {
+        if (p < 0) return;
+        const long long a = (long long)(p >> 16) * rc.W + (p & 0xffff);
+        if constexpr (STORED) fetch_window<G, S>(land, rc.win + a * kRec);
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(land + kRec);
+        if (lane == 30)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(rc.draw4 + a) : "memory");
+        if (lane == 31)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 16u), "l"(rc.draw1 + a) : "memory");
+    };
+    PixWin<S> pw;
+    bool o2_full = false;   // pw.o2 holds the offsets of a window wholly inside the image
+    unsigned nev = 0;
+    int next = take();
+    fetch(next);
+    while (next >= 0) {
+        const int px = next & 0xffff, py = next >> 16;
+        const long long pix = (long long)py * rc.W + px;
+        fetch_wait();
         __syncwarp();
+        if constexpr (STORED) {
+            const float2* wp = reinterpret_cast<const float2*>(land) + (lane & (G - 1));
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+                const float2 v = wp[s * G];
+                pw.w[s] = v.x;
+                pw.wr[s] = v.y;
+            }
+            pw.ok = land[2 * G * S + 12] != 0.0f;
+            if (lane < 12) reinterpret_cast<float*>(&ws->geo)[lane] = land[2 * G * S + lane];
+        }
+        if (lane < 5) ws->draw[lane] = land[kRec + lane];
+        __syncwarp();
+        next = take();
+        fetch(next);
+        if constexpr (STORED) {
+            if (!pw.ok) continue;   // flat patch: every hypothesis costs C_max
+            int ku_lo, ku_hi, kv_lo, kv_hi;
+            window_range(rc, px, py, ku_lo, ku_hi, kv_lo, kv_hi);
+            const bool full = ku_lo == 0 && kv_lo == 0 && ku_hi == rc.n - 1 && kv_hi == rc.n - 1;
+            if (!full || !o2_full) window_offsets<G, S>(rc, ku_lo, ku_hi, kv_lo, kv_hi, pw.o2);
+            o2_full = full;
+        } else {
+            build_window<G, S>(rc, px, py, true, pw);
+            if (!pw.ok) continue;
+            if (lane == 0) ws->geo = pw.geo;
+        }
+        // the pixel's state waits in shared memory (fewer live registers
+        // through the evaluation rounds)
         if (lane == 0) {
-            ws->geo = pw.geo;
             ws->cur = rc.plane[pix];
             ws->cur_c = rc.cost[pix];
         }
@@ -335,8 +422,8 @@ __global__ void __launch_bounds__(PhaseTile<S>::BLOCK, PhaseTile<S>::MIN_BLOCKS)
 
         // ---- propagation: lane g < 8 takes group g's cheapest member and
         // carries its plane over
-        int member;
-        const int q = best_members(rc, px, py, member);
+        int member, x2, y2;
+        const int q = best_members(rc, members, px, py, member, x2, y2);
         // candidate memo: group g's (member, plane generation) now and at this
         // pixel's last visit in this call; an unchanged one was scored then
         uint32_t key = 0xfffffffeu;
@@ -351,7 +438,6 @@ __global__ void __launch_bounds__(PhaseTile<S>::BLOCK, PhaseTile<S>::MIN_BLOCKS)
         if (ok) {
             // the neighbour's plane carried over as a plane (reading)
             np = rc.plane[q];
-            int x2 = q % rc.W, y2 = q / rc.W;
             const float* Ki = rc.Kinv;
             float r0 = fmaf(Ki[0], (float)x2, fmaf(Ki[1], (float)y2, Ki[2]));
             float r1 = fmaf(Ki[3], (float)x2, fmaf(Ki[4], (float)y2, Ki[5]));
@@ -366,15 +452,16 @@ __global__ void __launch_bounds__(PhaseTile<S>::BLOCK, PhaseTile<S>::MIN_BLOCKS)
         // plane or to an earlier group's plane scores the same cost, so it
         // cannot be strictly cheaper than that plane: it is not evaluated.
         {
-            const float4 mine = make_float4(np.x, np.y, np.z, d);
-            bool dup = ok && same_plane(mine, ws->cur);
-#pragma unroll
-            for (int g2 = 0; g2 < 7; ++g2) {
-                const float4 o = make_float4(__shfl_sync(0xffffffffu, np.x, g2), __shfl_sync(0xffffffffu, np.y, g2),
-                                             __shfl_sync(0xffffffffu, np.z, g2), __shfl_sync(0xffffffffu, d, g2));
-                const bool ook = __shfl_sync(0xffffffffu, (int)ok, g2) != 0;
-                dup = dup || (ok && ook && lane > g2 && same_plane(mine, o));
-            }
+            // lane b (b - 1) / 2 + a tests the pair of groups a < b (28 pairs)
+            if (lane < 8) ws->hyp[lane] = make_float4(np.x, np.y, np.z, ok ? d : __int_as_float(0x7fc00000));
+            __syncwarp();
+            const int b = 1 + (lane >= 1) + (lane >= 3) + (lane >= 6) + (lane >= 10) + (lane >= 15) + (lane >= 21);
+            const int a = min(lane - b * (b - 1) / 2, 7);
+            const unsigned eq = __ballot_sync(0xffffffffu, lane < 28 && same_plane(ws->hyp[b], ws->hyp[a]));
+            const int lb = lane & 7;
+            const bool dup = ok && (((eq >> (lb * (lb - 1) / 2)) & ((1u << lb) - 1u)) != 0u ||
+                                    same_plane(make_float4(np.x, np.y, np.z, d), ws->cur));
+            __syncwarp();
             ok = ok && !dup;
         }
         ok = ok && !repeat;
@@ -402,8 +489,8 @@ __global__ void __launch_bounds__(PhaseTile<S>::BLOCK, PhaseTile<S>::MIN_BLOCKS)
                 // the normal's angles theta = atan2(m1, m0), phi = acos(m2)
                 // (after flipping to m2 >= 0) move by delta_theta, delta_phi,
                 // taken through the angle-addition formulas
-                const float4 r4 = draw4[it & 31u];
-                const float sdp = draw1[it & 31u];
+                const float4 r4 = make_float4(ws->draw[0], ws->draw[1], ws->draw[2], ws->draw[3]);
+                const float sdp = ws->draw[4];
                 float d_new = fminf(fmaxf(cur.w + r4.x, rc.d_lo), rc.d_hi);
                 float m0 = cur.x, m1 = cur.y, m2 = cur.z;
                 if (m2 < 0.0f) { m0 = -m0; m1 = -m1; m2 = -m2; }
@@ -492,7 +579,8 @@ unsigned pm_grid_for(const void* kernel, long long units, size_t smem, int block
         if (it != cache.end() && it->second.smem == smem && it->second.block == block) {
             per_sm = it->second.per_sm;
         } else {
-            if (smem > 48 * 1024 &&
+            // 48 KB without the opt-in, static shared memory included
+            if (smem > 44 * 1024 &&
                 (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
                     cudaSuccess) {
                 t_grid_err = e;
@@ -549,9 +637,17 @@ static cudaError_t launch_status() {
             if (_h == 8) { CALL(8, 16); } else if (_h == 32) { CALL(32, 4); }             \
             else { CALL(16, 8); }                                                         \
         }                                                                                 \
-        else if (_s <= 256) { if (_h == 32) { CALL(32, 8); } else { CALL(16, 16); } }     \
-        else { CALL(32, 16); }                                                            \
+        else if (_s <= 256 && _h == 32) { CALL(32, 8); }                                  \
+        else { MVS_DISPATCH_DEFAULT(n, CALL); }                                           \
     } while (0)
+
+template <int G, int S, bool MX>
+const void* phase_kernel(const RefConst& rc) {
+    return rc.win ? (const void*)k_phase<G, S, MX, true> : (const void*)k_phase<G, S, MX, false>;
+}
+
+// floats of shared memory per phase warp for the stored windows
+static int phase_rec(const RefConst& rc, int G, int S) { return rc.win ? win_record_floats(G, S) : 0; }
 
 // Resolves (and caches) the grid sizes of the init / cost / phase kernels of
 // this configuration without launching anything, so that a later stream
@@ -562,9 +658,9 @@ cudaError_t prime_launch_configs(const RefConst& rc) {
     do {                                                                                              \
         pm_grid_for((const void*)k_init<G, S, MX>, 1, smem, kBlock);                                  \
         pm_grid_for((const void*)k_cost<G, S, MX>, 1, smem, kBlock);                                  \
-        pm_grid_for((const void*)k_phase<G, S, MX>, 1,                                                \
-                    phase_smem_bytes(rc.n_src, PhaseTile<S>::TX * phase_rows<S>(rc.n_src, MX), MX),  \
-                    32 * PhaseTile<S>::TX * phase_rows<S>(rc.n_src, MX));                              \
+        const int rec = phase_rec(rc, G, S), w = phase_warps<S>(rc.n_src, rec);                       \
+        pm_grid_for(phase_kernel<G, S, MX>(rc), 1, phase_smem_bytes(rc.n_src, w, rec), 32 * w);       \
+        if (rc.win) pm_grid_for((const void*)k_window<G, S>, 1, 0, kBlock);                            \
     } while (0)
     if (rc.precision) {
         constexpr bool MX = true;
@@ -585,12 +681,12 @@ cudaError_t launch_build_texture(const uint8_t* img, int W, int H, uint2* tex, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_init(const RefConst& rc, float* view_cost, cudaStream_t s) {
+cudaError_t launch_init(const RefConst& rc, cudaStream_t s) {
     long long npix = (long long)rc.W * rc.H;
     const size_t smem = smem_block_bytes(rc.n_src, kWarps);
     const unsigned units = (unsigned)((npix + kWarps - 1) / kWarps);
 #define CALL(G, S) \
-    k_init<G, S, MX><<<pm_grid_for((const void*)k_init<G, S, MX>, units, smem, kBlock), kBlock, smem, s>>>(rc, view_cost)
+    k_init<G, S, MX><<<pm_grid_for((const void*)k_init<G, S, MX>, units, smem, kBlock), kBlock, smem, s>>>(rc)
     if (rc.precision) {
         constexpr bool MX = true;
         MVS_DISPATCH_DEFAULT(rc.n, CALL);
@@ -622,21 +718,54 @@ cudaError_t launch_cost(const RefConst& rc, const float4* plane, float* cost, fl
     return launch_status();
 }
 
+// perturbations of an iteration (both colours)
+static void launch_draws(const RefConst& rc, int iter, cudaStream_t s) {
+    const long long n = (long long)rc.W * rc.H;
+    k_draws<<<(unsigned)std::min<long long>((n + 255) / 256, 152LL * 8), 256, 0, s>>>(rc, iter);
+    count_launch();
+}
+
 template <int G, int S, bool MX>
 void phase_launch(const RefConst& rc, int phase, cudaStream_t s) {
-    using T = PhaseTile<S>;
-    const int ty = phase_rows<S>(rc.n_src, MX), block = 32 * T::TX * ty;
-    const long long ntiles = (long long)(((rc.W + 1) / 2 + T::TX - 1) / T::TX) * ((rc.H + ty - 1) / ty);
-    const size_t smem = phase_smem_bytes(rc.n_src, T::TX * ty, MX);
-    k_phase<G, S, MX><<<pm_grid_for((const void*)k_phase<G, S, MX>, ntiles, smem, block), block, smem, s>>>(rc,
-                                                                                                           phase);
+    const int rec = phase_rec(rc, G, S), w = phase_warps<S>(rc.n_src, rec), block = 32 * w;
+    const long long ntiles = (long long)((rc.W + 1) / 2) * ((rc.H + kTileY - 1) / kTileY);
+    const size_t smem = phase_smem_bytes(rc.n_src, w, rec);
+    const unsigned grid = pm_grid_for(phase_kernel<G, S, MX>(rc), ntiles, smem, block);
+    if (rc.win) k_phase<G, S, MX, true><<<grid, block, smem, s>>>(rc, phase);
+    else k_phase<G, S, MX, false><<<grid, block, smem, s>>>(rc, phase);
+}
+
+size_t pm_window_bytes(const RefConst& rc) {
+    size_t b = 0;
+#define CALL(G, S) b = (size_t)win_record_floats(G, S) * sizeof(float)
+    if (rc.precision) {
+        MVS_DISPATCH_DEFAULT(rc.n, CALL);
+    } else {
+        MVS_DISPATCH(rc.n, rc.lanes_hint, CALL);
+    }
+#undef CALL
+    return b;
+}
+
+cudaError_t launch_windows(const RefConst& rc, cudaStream_t s) {
+    const unsigned units = (unsigned)(((long long)rc.W * rc.H + kWarps - 1) / kWarps);
+#define CALL(G, S) k_window<G, S><<<pm_grid_for((const void*)k_window<G, S>, units, 0, kBlock), kBlock, 0, s>>>(rc)
+    if (rc.precision) {
+        MVS_DISPATCH_DEFAULT(rc.n, CALL);
+    } else {
+        MVS_DISPATCH(rc.n, rc.lanes_hint, CALL);
+    }
+#undef CALL
+    count_launch();
+    return launch_status();
 }
 
 cudaError_t launch_memo_reset(const RefConst& rc, cudaStream_t s) {
     return cudaMemsetAsync(rc.memo, 0xff, (size_t)rc.W * rc.H * MVS_MEMO_WORDS * sizeof(uint32_t), s);
 }
 
-cudaError_t launch_phase(const RefConst& rc, int phase, cudaStream_t s) {
+cudaError_t launch_phase(const RefConst& rc, int phase, bool first, cudaStream_t s) {
+    if (first || (phase & 1) == 0) launch_draws(rc, phase >> 1, s);
     if (rc.precision) {
 #define CALL(G, S) phase_launch<G, S, true>(rc, phase, s)
         MVS_DISPATCH_DEFAULT(rc.n, CALL);
