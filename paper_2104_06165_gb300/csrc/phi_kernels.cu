@@ -653,7 +653,11 @@ cudaError_t launch_phi_hypotheses(int W, int H, const float* depth, const uint8_
         else if (_s <= 36) { CALL(4, 9); }          \
         else if (_s <= 64) { CALL(8, 8); }          \
         else if (_s <= 128) { CALL(16, 8); }        \
+        else if (_s <= 176) { CALL(16, 11); }       \
         else if (_s <= 256) { CALL(16, 16); }       \
+        else if (_s <= 320) { CALL(32, 10); }       \
+        else if (_s <= 384) { CALL(32, 12); }       \
+        else if (_s <= 448) { CALL(32, 14); }       \
         else { CALL(32, 16); }                      \
     } while (0)
 

@@ -612,8 +612,14 @@ static cudaError_t launch_status() {
     return g != cudaSuccess ? g : l;
 }
 
-// Lanes per pixel group (G) and slots per lane (S) for an n x n window:
-// G * S >= n * n.  lanes_hint 0 picks the default; 4, 8, 16 or 32 picks G.
+// Lanes per pixel group (G) and slots per lane (S) for an n x n window: the
+// smallest built G * S >= n * n, since an empty slot costs as much as a sample.
+// The dense windows get layouts of their own (768 x 513, 8 sources, 3
+// iterations): 13 x 13 on 16 x 11 instead of 16 x 16 slots 25.3 -> 13.8 ms,
+// 17 x 17 on 32 x 10 instead of 32 x 16 38.2 -> 21.6 ms, 19 x 19 on 32 x 12
+// 38.8 -> 25.3 ms, 21 x 21 on 32 x 14 39.5 -> 29.7 ms (15 x 15 keeps 16 x 16).
+// Slots past the window add exact zeros, so the results are the same bit for
+// bit.  lanes_hint 0 picks the default; 4, 8, 16 or 32 picks G.
 // The mixed-precision kernels exist for the default layout of each window
 // size only.
 #define MVS_DISPATCH_DEFAULT(n, CALL)                                                     \
@@ -623,7 +629,11 @@ static cudaError_t launch_status() {
         else if (_s <= 36) { CALL(4, 9); }                                                \
         else if (_s <= 64) { CALL(8, 8); }                                                \
         else if (_s <= 128) { CALL(16, 8); }                                              \
+        else if (_s <= 176) { CALL(16, 11); }                                             \
         else if (_s <= 256) { CALL(16, 16); }                                             \
+        else if (_s <= 320) { CALL(32, 10); }                                             \
+        else if (_s <= 384) { CALL(32, 12); }                                             \
+        else if (_s <= 448) { CALL(32, 14); }                                             \
         else { CALL(32, 16); }                                                            \
     } while (0)
 
