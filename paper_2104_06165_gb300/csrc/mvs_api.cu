@@ -62,6 +62,7 @@ struct mvs_ctx {
     std::vector<cudaEvent_t> ev;
     size_t ev_used = 0;
     long long launches0 = 0;
+    int* wait_status = nullptr;            // host memory the kernels write: MVS_DEV_TIMEOUT once a wait ran out
     unsigned long long* evals = nullptr;   // device counter of evaluated (pixel, hypothesis, view)
     // batched path
     cudaStream_t gstream = nullptr;        // private stream for graph capture / replay
@@ -130,6 +131,19 @@ void* scratch(mvs_ctx* c, int slot, size_t bytes, cudaError_t* e) {
     if (*e != cudaSuccess) { s.p = nullptr; return nullptr; }
     s.bytes = bytes;
     return s.p;
+}
+
+// MVS_ETIMEOUT once a bounded wait of this context's kernels ran out since the
+// last check: at the next call that uses them, or at once for host outputs
+mvs_status check_waits(mvs_ctx* c) {
+    if (!c->wait_status) {
+        CK(c, cudaHostAlloc((void**)&c->wait_status, sizeof(int), cudaHostAllocDefault));
+        *c->wait_status = 0;
+    }
+    volatile int* st = c->wait_status;
+    if (*st == 0) return MVS_OK;
+    *st = 0;
+    return fail(c, MVS_ETIMEOUT, "message passing gave up waiting for the row above");
 }
 
 // true when p is device (or managed) memory the kernels can read
@@ -363,6 +377,7 @@ void mvs_destroy(mvs_ctx* c) {
     for (auto& s : c->scratch) cudaFree(s.p);
     for (auto e : c->ev) cudaEventDestroy(e);
     cudaFree(c->evals);
+    cudaFreeHost(c->wait_status);
     for (auto& b : c->batch)
         if (b.exec) cudaGraphExecDestroy(b.exec);
     for (auto e : c->gev) if (e) cudaEventDestroy(e);
@@ -1068,6 +1083,8 @@ mvs_status mvs_phi_mrf(mvs_ctx* c, int32_t W, int32_t H, const uint8_t* known, c
         return fail(c, MVS_EINVAL, "need kappa1 > 0, kappa2 > 0, kappa3 > 1");
     if (mem != MVS_MEM_DEVICE && mem != MVS_MEM_HOST) return fail(c, MVS_EINVAL, "bad mem kind");
     CK(c, cudaSetDevice(c->device));
+    mvs_status ws = check_waits(c);
+    if (ws != MVS_OK) return ws;
     size_t n = (size_t)W * H;
     int gw = (W + 1) / 2, gh = (H + 1) / 2;
     size_t g = (size_t)gw * gh;
@@ -1097,10 +1114,11 @@ mvs_status mvs_phi_mrf(mvs_ctx* c, int32_t W, int32_t H, const uint8_t* known, c
         kd = k2; dd = d2; hd = h2; vd = v2; cd = c2; ld = l2;
     }
     CK(c, launch_phi_mrf(W, H, kd, dd, hd, vd, cd, phi->kappa1, phi->kappa2, phi->kappa3, phi->trw_iters, ld, work,
-                         c->stream));
+                         c->wait_status, c->stream));
     if (mem == MVS_MEM_HOST) {
         CK(c, cudaMemcpyAsync(label, ld, g * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
+        return check_waits(c);
     }
     return MVS_OK;
 }
@@ -1218,6 +1236,7 @@ mvs_status mvs_plane_infer(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t
     if (phi->selection != MVS_PHI_SELECT_MRF && phi->selection != MVS_PHI_SELECT_MIN_COST)
         return fail(c, MVS_EINVAL, "unknown selection %d", (int)phi->selection);
     CK(c, cudaSetDevice(c->device));
+    if ((st = check_waits(c)) != MVS_OK) return st;
     if ((st = ensure_map(c, ref)) != MVS_OK) return st;
     ViewData& V = c->views[ref];
     int W = V.cam.width, H = V.cam.height;
@@ -1257,12 +1276,15 @@ mvs_status mvs_plane_infer(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t
         CK(c, launch_phi_select_min_cost(rc, known, hyp, valid, hcost, V.plane, newd, c->stream));
     } else {
         CK(c, launch_phi_mrf(W, H, known, depth, hyp, valid, hcost, phi->kappa1, phi->kappa2, phi->kappa3,
-                             phi->trw_iters, label, mwork, c->stream));
+                             phi->trw_iters, label, mwork, c->wait_status, c->stream));
         CK(c, launch_phi_select(rc, known, hyp, valid, label, V.plane, newd, c->stream));
     }
     V.has_map = true;
     CK(c, cudaMemcpyAsync(inout->plane, V.plane, n * sizeof(float4), kind_out(mem), c->stream));
-    if (mem == MVS_MEM_HOST) CK(c, cudaStreamSynchronize(c->stream));
+    if (mem == MVS_MEM_HOST) {
+        CK(c, cudaStreamSynchronize(c->stream));
+        return check_waits(c);
+    }
     return MVS_OK;
 }
 

@@ -160,9 +160,10 @@ cudaError_t launch_phi_hypotheses(int W, int H, const float* depth, const uint8_
 cudaError_t phi_static_scratch(int32_t** out);
 cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t* valid, float* hcost,
                             cudaStream_t s);
+// status: a word both sides see; MVS_DEV_TIMEOUT once a wait between rows ran out
 cudaError_t launch_phi_mrf(int W, int H, const uint8_t* known, const float* depth, const float* hyp,
                            const uint8_t* valid, const float* hcost, float k1, float k2, float k3, int iters,
-                           int32_t* label, float* work, cudaStream_t s);
+                           int32_t* label, float* work, int* status, cudaStream_t s);
 size_t phi_mrf_work_floats(int W, int H);
 cudaError_t launch_phi_select(const RefConst& rc, const uint8_t* known, const float* hyp, const uint8_t* valid,
                               const int32_t* label, float4* plane, float* newdepth, cudaStream_t s);

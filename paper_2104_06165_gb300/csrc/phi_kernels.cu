@@ -2,8 +2,6 @@
 // (Sec. III-E): four-direction line-fit hypotheses, their matching cost, the
 // pairwise MRF of Eq. 6-9 decoded by tree-reweighted message passing at half
 // resolution, closest-hypothesis selection and Eq. 10 normals.
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <mutex>
 
@@ -240,28 +238,41 @@ __global__ void __launch_bounds__(kBlock, 3) k_phi_cost(const __grid_constant__ 
 // rows and columns as monotonic chains (node weight 1 / max(#earlier,
 // #later present neighbours)); one iteration = forward pass in raster order +
 // backward pass; decode = per-node argmin of the belief (lowest label on a
-// tie).  The raster order is run as anti-diagonal wavefronts (a node only
-// depends on its up / left neighbours in the forward pass and on its down /
-// right neighbours in the backward pass), which gives the same messages as
-// the sequential sweep.  One cooperative launch per pass pipelines strips of
-// kTrwRows node rows: a block owns strips b, b + gridDim.x, ... and walks each
-// in tiles of kTrwCols columns; at stage k strip s takes tile k - s, whose
-// upper neighbour tile (strip s - 1) was finished at stage k - 1 and whose
-// left neighbour tile by the same block at stage k - 1.  Stages are separated
-// by a grid barrier (ns + nb - 1 of them instead of gw + gh - 1), and the
-// anti-diagonals of a tile by a block barrier.  Inside a tile one warp takes
-// one node: lane (d, lq, l) evaluates the min-sum term of own label l towards
-// label lq of the d-th outgoing neighbour.  At the start of a stage the block
-// stages its tile in shared memory (unaries, label depths, the messages that
-// do not change during the pass, the messages entering the tile from the
-// tiles finished at the previous stage, written by other multiprocessors and
-// read at L2); inside the stage a message to the lower node passes through
-// shared memory and one to the right node stays in the warp's registers, so
-// the anti-diagonal steps wait on no global memory.  Every message is also
-// written to global memory (.cg) for the other pass and the decoding.  The
-// backward pass runs the same schedule on the mirrored grid.
+// tie).  A node depends on its up / left neighbours only (forward; on its down
+// / right ones in the backward pass, which runs the same schedule on the
+// mirrored grid), so the rows run as a pipeline with the messages of the
+// sequential sweep.
+//
+// What bounds it: a chain of gw + gh - 1 dependent nodes.  One warp walks one
+// row, lane (d, lq, l) evaluating the min-sum term of own label l towards
+// label lq of the d-th outgoing neighbour (down, right); the message to the
+// right stays in the warp's registers and the message down goes to the next
+// row's warp through a ring in shared memory (kTrwRows rows per block) or, at
+// the last row of a block, through global memory.  The data is its own flag:
+// an empty slot holds kTrwEmpty, a bit pattern no message has, so the reader
+// polls the words it needs and nothing else is signalled; the reader of a ring
+// slot empties it again and the writer finds it empty before it writes.
+// Blocks are co-resident (cooperative launch) and every poll is bounded.
+//
+// Work that does not depend on the messages stays out of the chain: the pair
+// energies of Eq. 7 come from a table (k_mrf_pairs), unaries and static
+// messages are fetched a chunk of 32 columns ahead, and a message to a node
+// with one label is zero (its only entry is its own minimum), so only nodes
+// with several labels and their neighbours are walked.
+//
+// 1536 x 1024 nodes, a quarter of them holes: 0.95 ms per pass against 5.43 ms
+// with 32 x 32 tiles and grid barriers (1.1 us per anti-diagonal: 32 warps of
+// one multiprocessor each evaluating the logarithms between block barriers);
+// all nodes holes 1.96 ms, none 0.03 ms.  A node takes about 0.3 us of a lone
+// warp's issue (0.6 us with eight rows waiting on one another); 12 rows per
+// block are the same within 1 %, 4 rows 4 % of the whole inference slower, and
+// one lane per (direction, label) over all own labels 10 % slower.
 // ---------------------------------------------------------------------------
-constexpr int kTrwRows = 32, kTrwCols = 32, kTrwBlock = 32 * kTrwRows;
+constexpr int kTrwRows = 8, kTrwCols = 32, kTrwRing = 128;
+constexpr uint32_t kTrwEmpty = 0xffffffffu;
+// polls per wait before it gives up (a few tenths of a second to a second;
+// a pass takes a millisecond)
+constexpr unsigned kTrwPolls = 1u << 23, kTrwPollsGlobal = 1u << 21;
 
 struct MrfBufs {
     int gw, gh;
@@ -270,6 +281,9 @@ struct MrfBufs {
     float* lab;       // [4] label depths
     float* un;        // [4] unary energies -log phi_n
     float* msg;       // [4 dir][4 lab] incoming messages (dir 0 up, 1 down, 2 left, 3 right)
+    float* pair;      // [2][4][4] Eq. 7 energies of (own label, neighbour's label): neighbour below, right
+    float* bnd;       // messages into the first row of each strip of kTrwRows rows: [strip][gw][4]
+    int* status;      // host-visible: MVS_DEV_TIMEOUT once a wait ran out
 };
 
 __global__ void k_mrf_setup(int W, int H, MrfBufs mb, const uint8_t* __restrict__ known,
@@ -280,22 +294,32 @@ __global__ void k_mrf_setup(int W, int H, MrfBufs mb, const uint8_t* __restrict_
     int gx = (int)(g % mb.gw), gy = (int)(g / mb.gw);
     long long i = (long long)(2 * gy) * W + 2 * gx;
     int L = 0;
+    float lab[4] = {0.f, 0.f, 0.f, 0.f}, un[4] = {0.f, 0.f, 0.f, 0.f};
+    int8_t lm[4] = {0, 0, 0, 0};
     if (known[i]) {
-        mb.lab[4 * g] = depth[i];
-        mb.un[4 * g] = 0.0f;
-        mb.lmap[4 * g] = -1;
+        lab[0] = depth[i];
+        lm[0] = -1;
         L = 1;
     } else {
+#pragma unroll
         for (int k = 0; k < 4; ++k)
             if (valid[4 * i + k]) {
-                mb.lab[4 * g + L] = hyp[4 * i + k];
-                mb.un[4 * g + L] = -logf((kCmax - hcost[4 * i + k]) / k1 + k2);   // Eq. 6
-                mb.lmap[4 * g + L] = (int8_t)k;
+                const float h = hyp[4 * i + k];
+                const float u = -logf((kCmax - hcost[4 * i + k]) / k1 + k2);   // Eq. 6
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q == L) { lab[q] = h; un[q] = u; lm[q] = (int8_t)k; }
                 L++;
             }
     }
+    reinterpret_cast<float4*>(mb.lab)[g] = make_float4(lab[0], lab[1], lab[2], lab[3]);
+    reinterpret_cast<float4*>(mb.un)[g] = make_float4(un[0], un[1], un[2], un[3]);
+    reinterpret_cast<char4*>(mb.lmap)[g] = make_char4(lm[0], lm[1], lm[2], lm[3]);
     mb.nlab[g] = (int8_t)L;
-    for (int k = 0; k < 16; ++k) mb.msg[16 * g + k] = 0.0f;
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4* m = reinterpret_cast<float4*>(mb.msg) + 4 * g;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = z;
 }
 
 // ((((a + b) + c) + d) + e): the belief sum in message-slot order
@@ -309,167 +333,266 @@ __device__ __forceinline__ float pair_energy(float h1, float h2, float k3) {
     return -2.0f * logf(k3 - fminf(1.0f, rel));
 }
 
-// Per-stage tile record in dynamic shared memory: the static data of the
-// tile's 32 x 32 nodes (pass-local row-major), of the targets just below and
-// right of it, the messages entering its first row and column from the
-// tiles finished at the previous stage, and the wavefront's downward
-// messages (double-buffered by step parity).
-struct TrwTileSm {
-    float4 un[kTrwRows * kTrwCols];    // unaries of the four labels
-    float4 lab[kTrwRows * kTrwCols];   // label depths
-    float4 msv[kTrwRows * kTrwCols];   // static message from the pass-local lower neighbour
-    float4 msh[kTrwRows * kTrwCols];   // static message from the pass-local right neighbour
-    float gamma[kTrwRows * kTrwCols];
-    int nl[kTrwRows * kTrwCols];       // labels (0: absent or outside the grid)
-    float4 lab_d[kTrwCols], lab_r[kTrwRows];   // targets below the last row / right of the last column
-    int nl_d[kTrwCols], nl_r[kTrwRows];
-    float4 up_b[kTrwCols], left_b[kTrwRows];   // messages into the first row / first column
-    float4 up_w[2][kTrwRows + 1];              // downward messages of the current wavefront
+// Pair energies of the edges whose messages are not trivially zero (one end
+// with several labels, the other present): thread (node, d, a) fills the four
+// entries of own label a towards the labels of the neighbour below (d 0) or
+// right (d 1).
+__global__ void k_mrf_pairs(MrfBufs mb, float k3) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long g = t >> 3;
+    if (g >= (long long)mb.gw * mb.gh) return;
+    const int d = (int)(t >> 2) & 1, a = (int)t & 3;
+    const int x = (int)(g % mb.gw), y = (int)(g / mb.gw);
+    if (d ? x + 1 >= mb.gw : y + 1 >= mb.gh) return;
+    const long long q = d ? g + 1 : g + mb.gw;
+    const int L = mb.nlab[g], Lq = mb.nlab[q];
+    if (a >= L || Lq < 1 || (L < 2 && Lq < 2)) return;
+    const float h = mb.lab[4 * g + a];
+    const float4 hq = reinterpret_cast<const float4*>(mb.lab)[q];
+    float4 o;
+    o.x = pair_energy(h, hq.x, k3);
+    o.y = Lq > 1 ? pair_energy(h, hq.y, k3) : 0.0f;
+    o.z = Lq > 2 ? pair_energy(h, hq.z, k3) : 0.0f;
+    o.w = Lq > 3 ? pair_energy(h, hq.w, k3) : 0.0f;
+    reinterpret_cast<float4*>(mb.pair)[t] = o;
+}
+
+// A warp's chunk of 32 columns.
+struct TrwChunk {
+    float un[kTrwCols * 4];    // unaries
+    float mv[kTrwCols * 4];    // static message from the pass-local lower neighbour
+    float mh[kTrwCols * 4];    // static message from the pass-local right neighbour
+    float mu[kTrwCols * 4];    // message from the upper neighbour if that has one label (else unused)
+    float ml[kTrwCols * 4];    // message from the left neighbour likewise
+    float gamma[kTrwCols];
+    uint32_t info[kTrwCols];   // labels of the node | lower << 8 | right << 16 | left neighbour << 24
+    float pair[kTrwCols * 32]; // the node's two pair-energy tables
+};
+// Shared memory of a block: per warp two chunks (the current and the next one's
+// pair tables) and the ring of messages into its row.
+struct TrwSm {
+    TrwChunk chunk[kTrwRows][2];
+    float ring[kTrwRows][kTrwRing * 4];
 };
 
-__global__ void __launch_bounds__(kTrwBlock, 1) k_trw_strips(MrfBufs mb, bool forward, float k3) {
-    cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+__global__ void __launch_bounds__(32 * kTrwRows, 1) k_trw_rows(MrfBufs mb, bool forward) {
     extern __shared__ __align__(16) unsigned char trw_smem[];
-    TrwTileSm& T = *reinterpret_cast<TrwTileSm*>(trw_smem);
+    TrwSm& sm = *reinterpret_cast<TrwSm*>(trw_smem);
+    __shared__ volatile int dead;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ns = (mb.gh + kTrwRows - 1) / kTrwRows, nb = (mb.gw + kTrwCols - 1) / kTrwCols;
+    if (tid == 0) dead = 0;
+    for (int i = tid; i < kTrwRows * kTrwRing * 4; i += blockDim.x)
+        (&sm.ring[0][0])[i] = __uint_as_float(kTrwEmpty);
+    __syncthreads();
+    const int ns = (mb.gh + kTrwRows - 1) / kTrwRows;
     // message slots (dir 0 up, 1 down, 2 left, 3 right) in pass-local terms:
     // the static ones come from the lower / right neighbours, the dynamic
     // ones from the upper / left neighbours updated earlier in this pass
-    const int sv = forward ? 1 : 0, sh = forward ? 3 : 2, dv = forward ? 0 : 1, dh = forward ? 2 : 3;
+    const int sv = forward ? 1 : 0, sh = forward ? 3 : 2;
     // original node index of pass-local (xf, yf), or -1 outside the grid
     auto node = [&](int xf, int yf) -> long long {
         if (xf < 0 || yf < 0 || xf >= mb.gw || yf >= mb.gh) return -1;
         const int x = forward ? xf : mb.gw - 1 - xf, y = forward ? yf : mb.gh - 1 - yf;
         return (long long)y * mb.gw + x;
     };
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = 0; k < ns + nb - 1; ++k) {
-        for (int st = blockIdx.x; st < ns; st += gridDim.x) {
-            const int c = k - st;
-            if (c < 0 || c >= nb) continue;              // block-uniform
-            const int x0 = c * kTrwCols, y0 = st * kTrwRows;
-            // ---- load the tile (one node per thread) and its borders
-            {
-                const int r = tid / kTrwCols, cc = tid % kTrwCols;
-                const long long i = node(x0 + cc, y0 + r);
-                int L = 0;
-                float gm = 1.0f;
-                float4 un = z4, lb = z4, mv = z4, mh = z4;
-                if (i >= 0) {
-                    L = mb.nlab[i];
-                    const int x = (int)(i % mb.gw), y = (int)(i / mb.gw);
-                    const int nbx[4] = {0, 0, -1, 1}, nby[4] = {-1, 1, 0, 0};
-                    int before = 0, after = 0;
+    auto labels = [&](long long i) { return i >= 0 ? (int)__ldg(mb.nlab + i) : 0; };
+    const int dsel = lane >> 4, lq = (lane >> 2) & 3, l = lane & 3;
+    const int dir = forward ? (dsel ? 3 : 1) : (dsel ? 2 : 0);
+    // entry (own label l, target's label lq) of a pair table: the table
+    // belongs to the upper / left end of the edge
+    const int pe_at = dsel * 16 + (forward ? l * 4 + lq : lq * 4 + l);
+    volatile float* ring_in = sm.ring[warp];
+    const bool to_ring = warp + 1 < kTrwRows;
+    volatile float* ring_out = sm.ring[to_ring ? warp + 1 : 0];
+
+    // each warp runs its row of every strip of the block, in order; row y
+    // waits for row y - 1 only, so the lowest unfinished row always advances
+    for (int st = blockIdx.x; st < ns; st += gridDim.x) {
+        const int yf = st * kTrwRows + warp;
+        if (yf >= mb.gh) break;
+        float* bnd_in = mb.bnd + (long long)st * mb.gw * 4;
+        float* bnd_out = bnd_in + (long long)mb.gw * 4;
+        const bool last_row = yf + 1 >= mb.gh;
+        float4 f_un, f_mv, f_mh, f_mu, f_ml;
+        float f_gm = 1.0f;
+        uint32_t f_info = 0;
+        int f_lu = 0;
+        // message to node i (L labels) from its pass-local upper (d 0) or left
+        // (d 1) neighbour q with one label: that neighbour's belief and the
+        // message into it are zero, so it is the pair energies less their
+        // minimum, whatever the pass; also stored for the other pass
+        auto from_known = [&](long long i, long long q, int d, int L) {
+            float v[4];
+            if (forward) {
+                const float4 t = reinterpret_cast<const float4*>(mb.pair)[8 * q + 4 * d];
+                v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+            } else {
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) {
-                        const int qx = x + nbx[d], qy = y + nby[d];
-                        const bool in = qx >= 0 && qx < mb.gw && qy >= 0 && qy < mb.gh;
-                        const int nq = in ? mb.nlab[(long long)qy * mb.gw + qx] : 0;
-                        if (nq > 0) { if (d == 0 || d == 2) before++; else after++; }
-                    }
-                    const int mx = max(before, after);
-                    gm = mx > 0 ? 1.0f / (float)mx : 1.0f;
-                    un = reinterpret_cast<const float4*>(mb.un)[i];
-                    lb = reinterpret_cast<const float4*>(mb.lab)[i];
-                    mv = __ldcg(reinterpret_cast<const float4*>(mb.msg + 16 * i + 4 * sv));
-                    mh = __ldcg(reinterpret_cast<const float4*>(mb.msg + 16 * i + 4 * sh));
-                }
-                T.nl[tid] = L;
-                T.gamma[tid] = gm;
-                T.un[tid] = un;
-                T.lab[tid] = lb;
-                T.msv[tid] = mv;
-                T.msh[tid] = mh;
-                if (tid < kTrwCols) {                     // targets below the tile
-                    const long long q = node(x0 + tid, y0 + kTrwRows);
-                    T.nl_d[tid] = q >= 0 ? mb.nlab[q] : 0;
-                    T.lab_d[tid] = q >= 0 ? reinterpret_cast<const float4*>(mb.lab)[q] : z4;
-                } else if (tid < kTrwCols + kTrwRows) {   // targets right of the tile
-                    const int rr = tid - kTrwCols;
-                    const long long q = node(x0 + kTrwCols, y0 + rr);
-                    T.nl_r[rr] = q >= 0 ? mb.nlab[q] : 0;
-                    T.lab_r[rr] = q >= 0 ? reinterpret_cast<const float4*>(mb.lab)[q] : z4;
-                } else if (tid < 2 * kTrwCols + kTrwRows) {   // into the first row (previous stage)
-                    const int c2 = tid - kTrwCols - kTrwRows;
-                    const long long q = node(x0 + c2, y0);
-                    T.up_b[c2] = q >= 0 ? __ldcg(reinterpret_cast<const float4*>(mb.msg + 16 * q + 4 * dv)) : z4;
-                } else if (tid < 2 * kTrwCols + 2 * kTrwRows) {   // into the first column
-                    const int r2 = tid - 2 * kTrwCols - kTrwRows;
-                    const long long q = node(x0, y0 + r2);
-                    T.left_b[r2] = q >= 0 ? __ldcg(reinterpret_cast<const float4*>(mb.msg + 16 * q + 4 * dh)) : z4;
+                for (int k = 0; k < 4; ++k) v[k] = k < L ? mb.pair[32 * i + 16 * d + 4 * k] : 0.0f;
+            }
+            float mn = 3.0e38f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (k < L) mn = fminf(mn, v[k]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = k < L ? v[k] - mn : 0.0f;
+            const float4 o = make_float4(v[0], v[1], v[2], v[3]);
+            __stcg(reinterpret_cast<float4*>(mb.msg + 16 * i + 4 * ((forward ? 0 : 1) + 2 * d)), o);
+            return o;
+        };
+        // lane c's node of the chunk at x0: into registers, and its pair
+        // tables into the chunk buffer in the background
+        auto fetch = [&](int x0, TrwChunk& C) {
+            const int xf = x0 + lane;
+            const long long i = node(xf, yf);
+            f_un = f_mv = f_mh = f_mu = f_ml = make_float4(0.f, 0.f, 0.f, 0.f);
+            f_info = 0;
+            f_gm = 1.0f;
+            f_lu = 0;
+            const int L = labels(i);
+            if (L >= 2) {
+                const long long qd = node(xf, yf + 1), qr = node(xf + 1, yf), qu = node(xf, yf - 1), ql = node(xf - 1, yf);
+                const int Ld = labels(qd), Lr = labels(qr), Lu = labels(qu), Ll = labels(ql);
+                const int mx = max((Lu > 0) + (Ll > 0), (Ld > 0) + (Lr > 0));
+                f_gm = mx > 0 ? 1.0f / (float)mx : 1.0f;
+                f_info = (uint32_t)L | ((uint32_t)Ld << 8) | ((uint32_t)Lr << 16) | ((uint32_t)Ll << 24);
+                f_lu = Lu;
+                f_un = reinterpret_cast<const float4*>(mb.un)[i];
+                f_mv = __ldcg(reinterpret_cast<const float4*>(mb.msg + 16 * i + 4 * sv));
+                f_mh = __ldcg(reinterpret_cast<const float4*>(mb.msg + 16 * i + 4 * sh));
+                if (Lu == 1) f_mu = from_known(i, qu, 0, L);
+                if (Ll == 1) f_ml = from_known(i, ql, 1, L);
+                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(C.pair + 32 * lane);
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    const long long o = forward ? i : (d ? qr : qd);   // the edge's upper / left end
+                    if ((d ? Lr : Ld) < 2) continue;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 64u * d + 16u * k),
+                                     "l"(mb.pair + 32 * o + 16 * d + 4 * k)
+                                     : "memory");
                 }
             }
-            __syncthreads();
-            // ---- the tile's anti-diagonals: warp = row, lane (dsel, lq, l)
-            // evaluates the min-sum term of own label l towards label lq of
-            // the lower (dsel 0) or right (dsel 1) neighbour
-            const int dsel = lane >> 4, lq = (lane >> 2) & 3, l = lane & 3;
-            const int dir = forward ? (dsel ? 3 : 1) : (dsel ? 2 : 0);
-            float left_in = 0.0f;                         // message from the left node, kept by this warp
-            for (int t = 0; t < kTrwRows + kTrwCols - 1; ++t) {
-                const int u = t - warp;                   // tile column of this warp's node
-                float out_v = 0.0f, out_h = 0.0f;         // messages sent down / right (0: none)
-                if (u >= 0 && u < kTrwCols) {
-                    const int n = warp * kTrwCols + u;
-                    const int L = T.nl[n];
-                    if (L > 0) {                          // warp-uniform
-                        const float4 un4 = T.un[n], mv4 = T.msv[n], mh4 = T.msh[n], lb4 = T.lab[n];
-                        const float unl = l == 0 ? un4.x : l == 1 ? un4.y : l == 2 ? un4.z : un4.w;
-                        const float mvl = l == 0 ? mv4.x : l == 1 ? mv4.y : l == 2 ? mv4.z : mv4.w;
-                        const float mhl = l == 0 ? mh4.x : l == 1 ? mh4.y : l == 2 ? mh4.z : mh4.w;
-                        const float labl = l == 0 ? lb4.x : l == 1 ? lb4.y : l == 2 ? lb4.z : lb4.w;
-                        const float4 upv = warp == 0 ? T.up_b[u] : T.up_w[(t - 1) & 1][warp];
-                        const float dynv = l == 0 ? upv.x : l == 1 ? upv.y : l == 2 ? upv.z : upv.w;
-                        float dynh = left_in;
-                        if (u == 0) {
-                            const float4 lf = T.left_b[warp];
-                            dynh = l == 0 ? lf.x : l == 1 ? lf.y : l == 2 ? lf.z : lf.w;
+        };
+        // warp 0: the words of the 8 columns from x8 that came from the strip
+        // above (lane = column, word)
+        auto peek = [&](int x8) {
+            const int x = x8 + (lane >> 2);
+            return x < mb.gw ? __ldcv(bnd_in + 4 * x + (lane & 3)) : 0.0f;
+        };
+        float left_in = 0.0f;             // message from the last node to its right neighbour
+        int seen8 = -1;                   // warp 0: the 8 columns that `seen` holds, all there
+        float seen = 0.0f, ahead = 0.0f;
+        fetch(0, sm.chunk[warp][0]);
+        if (warp == 0 && st > 0) ahead = peek(0);
+        int ahead8 = 0;
+        for (int x0 = 0; x0 < mb.gw; x0 += kTrwCols) {
+            TrwChunk& C = sm.chunk[warp][(x0 / kTrwCols) & 1];
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            reinterpret_cast<float4*>(C.un)[lane] = f_un;
+            reinterpret_cast<float4*>(C.mv)[lane] = f_mv;
+            reinterpret_cast<float4*>(C.mh)[lane] = f_mh;
+            reinterpret_cast<float4*>(C.mu)[lane] = f_mu;
+            reinterpret_cast<float4*>(C.ml)[lane] = f_ml;
+            C.gamma[lane] = f_gm;
+            C.info[lane] = f_info;
+            // the nodes with several labels, and those of them with a message
+            // from such a node of the row above
+            unsigned todo = __ballot_sync(0xffffffffu, f_info != 0);
+            const unsigned in_up = __ballot_sync(0xffffffffu, f_lu >= 2);
+            __syncwarp();
+            if (x0 + kTrwCols < mb.gw) fetch(x0 + kTrwCols, sm.chunk[warp][((x0 / kTrwCols) & 1) ^ 1]);
+            while (todo) {
+                const int c = __ffs(todo) - 1, x = x0 + c;
+                todo &= todo - 1u;
+                const uint32_t info = C.info[c];
+                const int L = info & 255, Ld = (info >> 8) & 255, Lr = (info >> 16) & 255;
+                const float unl = C.un[4 * c + l], mvl = C.mv[4 * c + l], mhl = C.mh[4 * c + l], gm = C.gamma[c];
+                const float pe = C.pair[32 * c + pe_at];
+                // (a left neighbour with several labels was this warp's last node)
+                const float dynh = (info >> 24) >= 2 ? left_in : C.ml[4 * c + l];
+                // ---- message from the row above
+                float dynv = C.mu[4 * c + l];
+                if ((in_up >> c) & 1u) {
+                    bool ok = false;
+                    if (warp > 0) {
+                        volatile float* slot = ring_in + 4 * (x & (kTrwRing - 1));
+                        for (unsigned it = 0; it < kTrwPolls; ++it) {
+                            dynv = slot[l];
+                            ok = __all_sync(0xffffffffu, __float_as_uint(dynv) != kTrwEmpty);
+                            if (ok || __any_sync(0xffffffffu, dead)) break;
                         }
-                        // belief of own label l: unary + the four incoming messages in slot order
-                        const float bel = forward ? un_add4(unl, dynv, mvl, dynh, mhl) : un_add4(unl, mvl, dynv, mhl, dynh);
-                        int Lq;
-                        float4 lq4;
-                        if (dsel == 0) {
-                            Lq = warp + 1 < kTrwRows ? T.nl[n + kTrwCols] : T.nl_d[u];
-                            lq4 = warp + 1 < kTrwRows ? T.lab[n + kTrwCols] : T.lab_d[u];
-                        } else {
-                            Lq = u + 1 < kTrwCols ? T.nl[n + 1] : T.nl_r[warp];
-                            lq4 = u + 1 < kTrwCols ? T.lab[n + 1] : T.lab_r[warp];
+                        if (lane < 4) slot[lane] = __uint_as_float(kTrwEmpty);
+                    } else {
+                        const int x8 = x & ~7;
+                        ok = true;
+                        if (seen8 != x8) {
+                            // every word of the 8 columns that will come
+                            const unsigned live8 = (in_up >> (x8 - x0)) & 255u;
+                            const bool want = (live8 >> (lane >> 2)) & 1u;
+                            seen = ahead8 == x8 ? ahead : peek(x8);
+                            for (unsigned it = 0; it < kTrwPollsGlobal; ++it) {
+                                ok = __all_sync(0xffffffffu, !want || __float_as_uint(seen) != kTrwEmpty);
+                                if (ok || __any_sync(0xffffffffu, dead)) break;
+                                seen = peek(x8);
+                            }
+                            seen8 = x8;
+                            ahead8 = x8 + 8;
+                            ahead = peek(ahead8);
                         }
-                        const float labq = lq == 0 ? lq4.x : lq == 1 ? lq4.y : lq == 2 ? lq4.z : lq4.w;
-                        const float mdir = dsel ? mhl : mvl;
-                        float e = 3.0e38f;
-                        if (l < L && lq < Lq) e = T.gamma[n] * bel - mdir + pair_energy(labl, labq, k3);
-                        // minimum over own labels, then over the target's labels (normalisation)
-                        e = fminf(e, __shfl_xor_sync(0xffffffffu, e, 1));
-                        e = fminf(e, __shfl_xor_sync(0xffffffffu, e, 2));
-                        float mn = fminf(e, __shfl_xor_sync(0xffffffffu, e, 4));
-                        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 8));
-                        const float o = lq < Lq ? e - mn : 0.0f;
-                        if (l == 0 && lq < Lq) {
-                            const long long q = dsel == 0 ? node(x0 + u, y0 + warp + 1) : node(x0 + u + 1, y0 + warp);
-                            __stcg(mb.msg + 16 * q + 4 * (dir ^ 1) + lq, o);
+                        dynv = __shfl_sync(0xffffffffu, seen, 4 * (x - x8) + l);
+                    }
+                    if (!ok) {
+                        if (lane == 0) {
+                            dead = 1;
+                            *reinterpret_cast<volatile int*>(mb.status) = MVS_DEV_TIMEOUT;
                         }
-                        // lane j < 4: the message to label j of the node below
-                        // (sent by lane 4 j); every lane: the message to label l
-                        // of the right node (sent by lane 16 + 4 l)
-                        out_v = __shfl_sync(0xffffffffu, o, 4 * l);
-                        out_h = __shfl_sync(0xffffffffu, o, 16 + 4 * l);
+                        return;
                     }
                 }
-                // the node below reads the downward message at the next step
-                // (lanes 0..3 write its four labels), the right node is this
-                // warp's next node
-                if (lane < 4) {
-                    float* w = reinterpret_cast<float*>(&T.up_w[t & 1][warp + 1]);
-                    w[lane] = out_v;
+                // ---- belief of own label l: unary + the four incoming messages in slot order
+                const float bel = forward ? un_add4(unl, dynv, mvl, dynh, mhl) : un_add4(unl, mvl, dynv, mhl, dynh);
+                const int Lq = dsel ? Lr : Ld;
+                float e = 3.0e38f;
+                if (l < L && lq < Lq && Lq >= 2) e = fmaf(gm, bel, -(dsel ? mhl : mvl)) + pe;
+                // minimum over own labels, then over the target's labels (normalisation)
+                e = fminf(e, __shfl_xor_sync(0xffffffffu, e, 1));
+                e = fminf(e, __shfl_xor_sync(0xffffffffu, e, 2));
+                float mn = fminf(e, __shfl_xor_sync(0xffffffffu, e, 4));
+                mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 8));
+                const float o = lq < Lq ? e - mn : 0.0f;
+                // lane j < 4: the message to label j of the node below (sent by
+                // lane 4 j); every lane: the message to label l of the right
+                // node (sent by lane 16 + 4 l)
+                left_in = __shfl_sync(0xffffffffu, o, 16 + 4 * l);
+                const float out_v = __shfl_sync(0xffffffffu, o, 4 * l);
+                if (Ld >= 2 && !last_row) {
+                    if (to_ring) {
+                        volatile float* slot = ring_out + 4 * (x & (kTrwRing - 1));
+                        bool ok = false;
+                        for (unsigned it = 0; it < kTrwPolls; ++it) {
+                            ok = __all_sync(0xffffffffu, lane >= 4 || __float_as_uint(slot[lane & 3]) == kTrwEmpty);
+                            if (ok || __any_sync(0xffffffffu, dead)) break;
+                        }
+                        if (!ok) {
+                            if (lane == 0) {
+                                dead = 1;
+                                *reinterpret_cast<volatile int*>(mb.status) = MVS_DEV_TIMEOUT;
+                            }
+                            return;
+                        }
+                        if (lane < 4) slot[lane] = out_v;
+                    } else if (lane < 4) {
+                        __stcg(bnd_out + 4 * x + lane, out_v);
+                    }
                 }
-                left_in = out_h;
-                __syncthreads();
+                if (l == 0 && lq < Lq && Lq >= 2) {
+                    const long long q = dsel == 0 ? node(x, yf + 1) : node(x + 1, yf);
+                    __stcg(mb.msg + 16 * q + 4 * (dir ^ 1) + lq, o);
+                }
             }
         }
-        grid.sync();                                      // every block runs the same number of stages
     }
 }
 
@@ -675,13 +798,14 @@ cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t*
 
 size_t phi_mrf_work_floats(int W, int H) {
     size_t g = (size_t)((W + 1) / 2) * ((H + 1) / 2);
-    // msg 16, lab 4, un 4 floats; nlab 1 + lmap 4 bytes (rounded up to 2 floats)
-    return g * (16 + 4 + 4 + 2) + 64;
+    const size_t strips = ((size_t)(H + 1) / 2 + kTrwRows - 1) / kTrwRows;
+    // msg 16, lab 4, un 4, pair 32 floats; nlab 1 + lmap 4 bytes (rounded up to 2 floats); strip boundaries
+    return g * (16 + 4 + 4 + 32 + 2) + strips * ((size_t)(W + 1) / 2) * 4 + 64;
 }
 
 cudaError_t launch_phi_mrf(int W, int H, const uint8_t* known, const float* depth, const float* hyp,
                            const uint8_t* valid, const float* hcost, float k1, float k2, float k3, int iters,
-                           int32_t* label, float* work, cudaStream_t s) {
+                           int32_t* label, float* work, int* status, cudaStream_t s) {
     MrfBufs mb;
     mb.gw = (W + 1) / 2;
     mb.gh = (H + 1) / 2;
@@ -689,12 +813,21 @@ cudaError_t launch_phi_mrf(int W, int H, const uint8_t* known, const float* dept
     mb.msg = work;
     mb.lab = mb.msg + 16 * g;
     mb.un = mb.lab + 4 * g;
-    mb.lmap = (int8_t*)(mb.un + 4 * g);
+    mb.pair = mb.un + 4 * g;
+    const long long ns = (mb.gh + kTrwRows - 1) / kTrwRows;
+    mb.bnd = mb.pair + 32 * g;
+    mb.lmap = (int8_t*)(mb.bnd + 4 * ns * mb.gw);
     mb.nlab = mb.lmap + 4 * g;
+    mb.status = status;
     k_mrf_setup<<<blocks_for(g, 256), 256, 0, s>>>(W, H, mb, known, depth, hyp, valid, hcost, k1, k2);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    if (iters > 0) {
+        k_mrf_pairs<<<blocks_for(8 * g, 256), 256, 0, s>>>(mb, k3);
+        count_launch();
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     // one block per strip, at most as many as are co-resident; the shared-
     // memory opt-in and the occupancy belong to the current device
     int max_blocks = 0;
@@ -708,24 +841,24 @@ cudaError_t launch_phi_mrf(int W, int H, const uint8_t* known, const float* dept
         if (!per_dev[dev]) {
             int sms = 0, per_sm = 0;
             if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            if ((e = cudaFuncSetAttribute(k_trw_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)sizeof(TrwTileSm))) != cudaSuccess)
+            if ((e = cudaFuncSetAttribute(k_trw_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)sizeof(TrwSm))) != cudaSuccess)
                 return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trw_strips, kTrwBlock,
-                                                                   sizeof(TrwTileSm))) != cudaSuccess)
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trw_rows, 32 * kTrwRows,
+                                                                   sizeof(TrwSm))) != cudaSuccess)
                 return e;
             if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
             per_dev[dev] = sms * per_sm;
         }
         max_blocks = per_dev[dev];
     }
-    const int want = (mb.gh + kTrwRows - 1) / kTrwRows;
-    dim3 grid(std::max(1, std::min(want, max_blocks))), block(kTrwBlock);
+    dim3 grid((unsigned)std::max<long long>(1, std::min<long long>(ns, max_blocks))), block(32 * kTrwRows);
     for (int it = 0; it < iters; ++it)
         for (int pass = 0; pass < 2; ++pass) {
             bool forward = pass == 0;
-            void* args[] = {(void*)&mb, (void*)&forward, (void*)&k3};
-            e = cudaLaunchCooperativeKernel((const void*)k_trw_strips, grid, block, args, sizeof(TrwTileSm), s);
+            void* args[] = {(void*)&mb, (void*)&forward};
+            if ((e = cudaMemsetAsync(mb.bnd, 0xff, sizeof(float) * 4 * ns * mb.gw, s)) != cudaSuccess) return e;
+            e = cudaLaunchCooperativeKernel((const void*)k_trw_rows, grid, block, args, sizeof(TrwSm), s);
             count_launch();
             if (e != cudaSuccess) return e;
         }
