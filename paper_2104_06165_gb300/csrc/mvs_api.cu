@@ -993,7 +993,7 @@ mvs_status mvs_phi_hypotheses(mvs_ctx* c, int32_t W, int32_t H, const float* dep
     CK(c, cudaSetDevice(c->device));
     size_t n = (size_t)W * H;
     cudaError_t e;
-    int32_t* work = (int32_t*)scratch(c, 1, n * 8 * sizeof(int32_t), &e);
+    int32_t* work = (int32_t*)scratch(c, 1, phi_line_words(W, H) * sizeof(uint32_t), &e);
     CK(c, e);
     const float* dd = depth;
     const uint8_t* kd = known;
@@ -1064,7 +1064,7 @@ mvs_status mvs_phi_cost(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t n_
         hd = h2;
         vd = v2;
     }
-    CK(c, launch_phi_cost(rc, hd, vd, cd, c->stream));
+    CK(c, launch_phi_cost(rc, hd, vd, cd, 1, c->stream));
     if (mem == MVS_MEM_HOST) {
         CK(c, cudaMemcpyAsync(hcost, cd, n * 4 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
@@ -1257,7 +1257,7 @@ mvs_status mvs_plane_infer(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t
     float* newd = depth + n;
     int32_t* label = (int32_t*)(newd + n);
     uint8_t* known = (uint8_t*)(label + g);
-    int32_t* work = (int32_t*)scratch(c, 1, n * 8 * sizeof(int32_t), &e);
+    int32_t* work = (int32_t*)scratch(c, 1, phi_line_words(W, H) * sizeof(uint32_t), &e);
     CK(c, e);
     float* mwork = (float*)scratch(c, 2, phi_mrf_work_floats(W, H) * sizeof(float), &e);
     CK(c, e);
@@ -1271,7 +1271,8 @@ mvs_status mvs_plane_infer(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t
     make_refconst(c, ref, srcs, n_src, pm, rc);
     CK(c, launch_phi_hypotheses(W, H, depth, known, phi->n_fit, phi->fit_inverse, pm->d_lo, pm->d_hi, hyp, valid,
                                 work, c->stream));
-    CK(c, launch_phi_cost(rc, hyp, valid, hcost, c->stream));
+    // the MRF's nodes are the even rows and columns; nothing else reads its costs
+    CK(c, launch_phi_cost(rc, hyp, valid, hcost, phi->selection == MVS_PHI_SELECT_MRF ? 2 : 1, c->stream));
     if (phi->selection == MVS_PHI_SELECT_MIN_COST) {
         CK(c, launch_phi_select_min_cost(rc, known, hyp, valid, hcost, V.plane, newd, c->stream));
     } else {

@@ -158,7 +158,9 @@ cudaError_t launch_phi_hypotheses(int W, int H, const float* depth, const uint8_
                                   float d_lo, float d_hi, float* hyp, uint8_t* valid, int32_t* scratch,
                                   cudaStream_t s);
 cudaError_t phi_static_scratch(int32_t** out);
-cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t* valid, float* hcost,
+size_t phi_line_words(int W, int H);   // scratch of launch_phi_hypotheses, 32-bit words
+// costs of the hypotheses of every step-th row and column (1: all pixels)
+cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t* valid, float* hcost, int step,
                             cudaStream_t s);
 // status: a word both sides see; MVS_DEV_TIMEOUT once a wait between rows ran out
 cudaError_t launch_phi_mrf(int W, int H, const uint8_t* known, const float* depth, const float* hyp,

@@ -85,113 +85,211 @@ __global__ void k_geo_filter(const __grid_constant__ FilterConst fc, uint8_t* __
 
 // ---------------------------------------------------------------------------
 // Sec. III-E hypotheses.  Direction k: 0 horizontal (1,0), 1 vertical (0,1),
-// 2 diagonal 45 deg below (1,1), 3 diagonal 45 deg above (1,-1).  A line of
-// direction k is indexed by its first pixel; gap[k][side][p] holds the
-// distance in steps from p to the nearest reconstructed pixel strictly
-// before (side 0) or after (side 1) p along the line, 0 if there is none.
+// 2 diagonal 45 deg below (1,1), 3 diagonal 45 deg above (1,-1).  The
+// reconstructed pixels are packed into bits along each direction, so that a
+// pixel finds its neighbours on a line by scanning words (32 pixels per load,
+// the next ones usually in the same word) instead of following per-pixel
+// distances that a thread per line wrote walking it (1.70 ms of serial walks
+// and 200 MB of distances at 3072 x 2048; the four bit maps and their summaries
+// take 3.5 MB and 0.19 ms).  Bit `pos` of line `li` is word [pos / 32][li] for the
+// directions 1-3 (adjacent pixels read adjacent words) and [li][pos / 32]
+// along the rows.  The position is x for direction 0, else y (x for the
+// diagonals of images more than 32 times as high as wide, which keeps the maps
+// within 8 words per pixel at any shape); lines are numbered y, x, x - y +
+// H - 1, x + y.
 // ---------------------------------------------------------------------------
 __constant__ int c_dir[4][2] = {{1, 0}, {0, 1}, {1, 1}, {1, -1}};
 
-__device__ __forceinline__ int n_lines(int k, int W, int H) { return k == 0 ? H : (k == 1 ? W : W + H - 1); }
-
-// start pixel of line l of direction k
-__device__ __forceinline__ void line_start(int k, int l, int W, int H, int& x, int& y) {
-    if (k == 0) { x = 0; y = l; }
-    else if (k == 1) { x = l; y = 0; }
-    else if (k == 2) {          // step (1,1): starts on the left column (bottom up) then the top row
-        if (l < H) { x = 0; y = H - 1 - l; } else { x = l - H + 1; y = 0; }
-    } else {                    // step (1,-1): starts on the left column then the bottom row
-        if (l < H) { x = 0; y = l; } else { x = l - H + 1; y = H - 1; }
-    }
-}
-
-__global__ void k_line_gaps(int W, int H, const uint8_t* __restrict__ known, int32_t* __restrict__ gaps) {
-    const long long N = (long long)W * H;
-    int k = blockIdx.y;
-    int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= n_lines(k, W, H)) return;
-    int sx = c_dir[k][0], sy = c_dir[k][1];
-    int x0, y0;
-    line_start(k, l, W, H, x0, y0);
-    int32_t* before = gaps + (long long)(2 * k) * N;
-    int32_t* after = gaps + (long long)(2 * k + 1) * N;
-    // forward walk: distance to the previous reconstructed pixel
-    int last = -1, t = 0;
-    for (int x = x0, y = y0; x >= 0 && x < W && y >= 0 && y < H; x += sx, y += sy, ++t) {
-        long long p = (long long)y * W + x;
-        before[p] = last >= 0 ? t - last : 0;
-        if (known[p]) last = t;
-    }
-    // backward walk: distance to the next reconstructed pixel
-    int len = t;
-    last = -1;
-    for (int s = len - 1; s >= 0; --s) {
-        int x = x0 + s * sx, y = y0 + s * sy;
-        long long p = (long long)y * W + x;
-        after[p] = last >= 0 ? last - s : 0;
-        if (known[p]) last = s;
-    }
-}
-
-// least-squares line v = a + b t through the n_fit reconstructed pixels
-// nearest along the line (negative side first at equal distance), value at
-// t = 0; centred normal equations in float
-__global__ void k_line_fit(int W, int H, const float* __restrict__ depth, const uint8_t* __restrict__ known,
-                           const int32_t* __restrict__ gaps, int n_fit, int inverse, float d_lo, float d_hi,
-                           float* __restrict__ hyp, uint8_t* __restrict__ valid) {
-    const long long N = (long long)W * H;
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    int x = (int)(i % W), y = (int)(i / W);
-    bool hole = !known[i];
+struct LineMaps {
+    int W, H, nwx, nwp;        // words per row; words per diagonal
+    bool along_y;              // the diagonals' position is y
+    uint32_t* bits[4];
+    uint32_t* sum[4];          // bit w of a line's summary: word w of the line is not empty
+    __host__ __device__ int lines(int k) const { return k == 0 ? H : (k == 1 ? W : W + H - 1); }
+    __host__ __device__ int words(int k) const { return k == 0 ? nwx : (k == 1 ? (H + 31) / 32 : nwp); }
+};
+__host__ __device__ inline LineMaps line_maps(int W, int H, uint32_t* base) {
+    LineMaps m;
+    m.W = W;
+    m.H = H;
+    m.nwx = (W + 31) / 32;
+    m.along_y = H / 32 <= W;
+    m.nwp = ((m.along_y ? H : W) + 31) / 32;
     for (int k = 0; k < 4; ++k) {
-        float h = 0.0f;
-        bool ok = false;
-        if (hole) {
-            const int32_t* before = gaps + (long long)(2 * k) * N;
-            const int32_t* after = gaps + (long long)(2 * k + 1) * N;
-            int sx = c_dir[k][0], sy = c_dir[k][1];
-            int dl = before[i], dr = after[i];   // distances of the next candidates on each side (0 = none)
-            float ts[32], vs[32];
-            int m = 0;
-            float tsum = 0.0f;
-            while (m < n_fit && (dl > 0 || dr > 0)) {
-                bool take_left = dl > 0 && (dr == 0 || dl <= dr);
-                int dist = take_left ? dl : dr;
-                int side = take_left ? -1 : 1;
-                long long q = (long long)(y + side * dist * sy) * W + (x + side * dist * sx);
-                float dv = depth[q];
-                ts[m] = (float)(side * dist);
-                vs[m] = inverse ? 1.0f / dv : dv;
-                tsum += ts[m];
-                m++;
-                if (take_left) {
-                    int g = before[q];
-                    dl = g > 0 ? dl + g : 0;
-                } else {
-                    int g = after[q];
-                    dr = g > 0 ? dr + g : 0;
-                }
+        m.bits[k] = base;
+        base += (size_t)m.lines(k) * m.words(k);
+    }
+    for (int k = 0; k < 4; ++k) {
+        m.sum[k] = base;
+        base += (size_t)m.lines(k) * ((m.words(k) + 31) / 32);
+    }
+    return m;
+}
+size_t line_map_words(int W, int H) {
+    const LineMaps m = line_maps(W, H, nullptr);
+    size_t n = 0;
+    for (int k = 0; k < 4; ++k) n += (size_t)m.lines(k) * (m.words(k) + (m.words(k) + 31) / 32);
+    return n;
+}
+
+// blockIdx.y = direction; direction 0: one warp per word, else one thread
+__global__ void k_line_bits(LineMaps m, const uint8_t* __restrict__ known) {
+    const int k = blockIdx.y, W = m.W, H = m.H;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0) {
+        const long long w = t >> 5;
+        if (w >= (long long)H * m.nwx) return;
+        const int y = (int)(w / m.nwx), x = (int)(w % m.nwx) * 32 + (int)(t & 31);
+        const unsigned b = __ballot_sync(0xffffffffu, x < W && known[(long long)y * W + x] != 0);
+        if ((t & 31) == 0) m.bits[0][w] = b;
+        return;
+    }
+    const int lines = m.lines(k), nw = m.words(k);
+    if (t >= (long long)lines * nw) return;
+    const int li = (int)(t % lines), p0 = (int)(t / lines) * 32;
+    uint32_t b = 0;
+#pragma unroll 8
+    for (int i = 0; i < 32; ++i) {
+        int x, y;
+        if (k == 1) {
+            x = li;
+            y = p0 + i;
+        } else {
+            const int c = k == 2 ? li - (H - 1) : li;   // x - y, x + y
+            if (m.along_y) {
+                y = p0 + i;
+                x = k == 2 ? c + y : c - y;
+            } else {
+                x = p0 + i;
+                y = k == 2 ? x - c : c - x;
             }
-            if (m >= 2) {
-                float tm = tsum / (float)m, vm = 0.0f;
-                for (int a = 0; a < m; ++a) vm += vs[a];
-                vm /= (float)m;
-                float stt = 0.0f, stv = 0.0f;
-                for (int a = 0; a < m; ++a) {
+        }
+        if (x >= 0 && x < W && y >= 0 && y < H && known[(long long)y * W + x]) b |= 1u << i;
+    }
+    m.bits[k][t] = b;
+}
+
+__global__ void k_line_sums(LineMaps m) {
+    const int k = blockIdx.y, lines = m.lines(k), nw = m.words(k), ns = (nw + 31) / 32;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)lines * ns) return;
+    // direction 0: [line][word], else [word][line]
+    const int li = (int)(k == 0 ? t / ns : t % lines), w0 = (int)(k == 0 ? t % ns : t / lines) * 32;
+    uint32_t b = 0;
+#pragma unroll 8
+    for (int i = 0; i < 32; ++i)
+        if (w0 + i < nw && m.bits[k][k == 0 ? (long long)li * nw + w0 + i : (long long)(w0 + i) * lines + li]) b |= 1u << i;
+    m.sum[k][t] = b;
+}
+
+// One side of a line: set bits strictly below (up = false) or above `pos`, in
+// order of distance; empty words are skipped through the summary, 32 at a time.
+struct LineScan {
+    const uint32_t* base;
+    const uint32_t* sums;
+    long long stride, sum_stride;
+    int ns, w, sw;             // summary words; current word and summary word
+    uint32_t word, sum;        // bits of word w, and of the summary past w, not taken yet
+    bool up;
+    // distance of the next reconstructed pixel from `pos`, 0 if there is none
+    __device__ __forceinline__ int next(int pos) {
+        if (!word) {
+            while (!sum) {
+                sw += up ? 1 : -1;
+                if (sw < 0 || sw >= ns) return 0;
+                sum = __ldg(sums + sw * sum_stride);
+            }
+            const int b = up ? __ffs(sum) - 1 : 31 - __clz(sum);
+            sum ^= 1u << b;
+            w = 32 * sw + b;
+            word = __ldg(base + w * stride);
+        }
+        const int b = up ? __ffs(word) - 1 : 31 - __clz(word);
+        word ^= 1u << b;
+        return up ? 32 * w + b - pos : pos - (32 * w + b);
+    }
+};
+
+// least-squares line v = a + b t through the n_fit <= NF reconstructed pixels
+// nearest along the line (negative side first at equal distance), value at
+// t = 0; centred normal equations in float.  One thread per pixel and
+// direction.
+template <int NF>
+__global__ void k_line_fit(LineMaps lm, const float* __restrict__ depth, const uint8_t* __restrict__ known, int n_fit,
+                           int inverse, float d_lo, float d_hi, float* __restrict__ hyp, uint8_t* __restrict__ valid) {
+    const int W = lm.W, H = lm.H;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long i = t >> 2;
+    const int k = (int)t & 3;
+    if (i >= (long long)W * H) return;
+    float h = 0.0f;
+    bool ok = false;
+    if (!known[i]) {
+        const int x = (int)(i % W), y = (int)(i / W);
+        const int sx = c_dir[k][0], sy = c_dir[k][1];
+        const int li = k == 0 ? y : (k == 1 ? x : (k == 2 ? x - y + H - 1 : x + y));
+        const int pos = k == 0 || (k >= 2 && !lm.along_y) ? x : y;
+        // along direction 3 with the position y, "before" is towards larger y
+        const bool flip = k == 3 && lm.along_y;
+        LineScan before, after;
+        const int lines = lm.lines(k), nw = lm.words(k), ns = (nw + 31) / 32;
+        before.base = lm.bits[k] + (k == 0 ? (long long)li * nw : li);
+        before.sums = lm.sum[k] + (k == 0 ? (long long)li * ns : li);
+        before.stride = before.sum_stride = k == 0 ? 1 : lines;
+        before.ns = ns;
+        before.w = pos >> 5;
+        before.sw = pos >> 10;
+        const uint32_t w0 = __ldg(before.base + before.w * before.stride);
+        const uint32_t s0 = __ldg(before.sums + before.sw * before.sum_stride);
+        after = before;
+        before.up = flip;
+        after.up = !flip;
+        auto below = [](uint32_t v, int b) { return v & ((1u << b) - 1u); };
+        auto above = [](uint32_t v, int b) { return v & ~((2u << b) - 1u); };
+        const int pb = pos & 31, wb = before.w & 31;
+        before.word = flip ? above(w0, pb) : below(w0, pb);
+        before.sum = flip ? above(s0, wb) : below(s0, wb);
+        after.word = flip ? below(w0, pb) : above(w0, pb);
+        after.sum = flip ? below(s0, wb) : above(s0, wb);
+        int dl = before.next(pos), dr = after.next(pos);   // distances of the next candidates on each side (0 = none)
+        float ts[NF], vs[NF];
+        int m = 0;
+        float tsum = 0.0f;
+#pragma unroll
+        for (int a = 0; a < NF; ++a) {
+            if (a >= n_fit || (dl == 0 && dr == 0)) break;
+            const bool take_left = dl > 0 && (dr == 0 || dl <= dr);
+            const int off = take_left ? -dl : dr;
+            const float dv = depth[(long long)(y + off * sy) * W + (x + off * sx)];
+            ts[a] = (float)off;
+            vs[a] = inverse ? 1.0f / dv : dv;
+            tsum += ts[a];
+            m++;
+            if (take_left) dl = before.next(pos);
+            else dr = after.next(pos);
+        }
+        if (m >= 2) {
+            float tm = tsum / (float)m, vm = 0.0f;
+#pragma unroll
+            for (int a = 0; a < NF; ++a)
+                if (a < m) vm += vs[a];
+            vm /= (float)m;
+            float stt = 0.0f, stv = 0.0f;
+#pragma unroll
+            for (int a = 0; a < NF; ++a)
+                if (a < m) {
                     float dt = ts[a] - tm;
                     stt = fmaf(dt, dt, stt);
                     stv = fmaf(dt, vs[a] - vm, stv);
                 }
-                float b = stv / stt;
-                float av = vm - b * tm;
-                h = inverse ? 1.0f / av : av;
-                ok = h >= d_lo && h <= d_hi;
-            }
+            float b = stv / stt;
+            float av = vm - b * tm;
+            h = inverse ? 1.0f / av : av;
+            ok = h >= d_lo && h <= d_hi;
         }
-        hyp[4 * i + k] = ok ? h : 0.0f;
-        valid[4 * i + k] = ok ? 1 : 0;
     }
+    hyp[t] = ok ? h : 0.0f;
+    valid[t] = ok ? 1 : 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -200,23 +298,29 @@ __global__ void k_line_fit(int W, int H, const float* __restrict__ depth, const 
 constexpr int kBlock = 128;
 constexpr int kWarps = kBlock / 32;
 
-// one warp per pixel, the four hypotheses of a pixel in lanes 0..3
+// One warp per pixel of the grid of every `step`-th row and column (the MRF
+// reads the costs at half resolution, so the inference scores those only), the
+// four hypotheses of a pixel in lanes 0..3.  5 blocks per SM (96 registers) as
+// in the other kernels of one visit per pixel.
 template <int G, int S>
-__global__ void __launch_bounds__(kBlock, 3) k_phi_cost(const __grid_constant__ RefConst rc, const float* __restrict__ hyp,
-                                                      const uint8_t* __restrict__ valid, float* __restrict__ hcost) {
+__global__ void __launch_bounds__(kBlock, S <= 9 ? 5 : S <= 11 ? 4 : 3)
+    k_phi_cost(const __grid_constant__ RefConst rc, const float* __restrict__ hyp, const uint8_t* __restrict__ valid,
+               float* __restrict__ hcost, int step) {
     extern __shared__ __align__(16) unsigned char smem[];
     ViewSm* views = reinterpret_cast<ViewSm*>(smem);
     load_views(rc, views);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long npix = (long long)rc.W * rc.H;
+    const int Ws = (rc.W + step - 1) / step, Hs = (rc.H + step - 1) / step;
+    const long long npix = (long long)Ws * Hs;
     unsigned nev = 0;
-    for (long long a = (long long)blockIdx.x * kWarps + warp; a < npix; a += (long long)gridDim.x * kWarps) {
+    for (long long b = (long long)blockIdx.x * kWarps + warp; b < npix; b += (long long)gridDim.x * kWarps) {
+        const int px = (int)(b % Ws) * step, py = (int)(b / Ws) * step;
+        const long long a = (long long)py * rc.W + px;
         bool v = lane < 4 && valid[4 * a + lane] != 0;
         if (!__any_sync(0xffffffffu, v)) {
             if (lane < 4) hcost[4 * a + lane] = kCmax;
             continue;
         }
-        const int px = (int)(a % rc.W), py = (int)(a / rc.W);
         PixWin<S> pw;
         build_window<G, S>(rc, px, py, true, pw);
         float h = lane < 4 ? hyp[4 * a + lane] : 1.0f;
@@ -728,8 +832,8 @@ cudaError_t launch_geo_filter(const FilterConst& fc, uint8_t* keep, int32_t* cou
     return cudaGetLastError();
 }
 
-// Fixed line-gap scratch of mvs_phi_hypotheses_static: 8 int32 per pixel for
-// up to MVS_PHI_STATIC_MAX_PIXELS pixels, in the library's own device memory.
+// Fixed line-map scratch of mvs_phi_hypotheses_static: 8 words per pixel (no
+// shape of an image needs more, see LineMaps) for up to MVS_PHI_STATIC_MAX_PIXELS pixels, in the library's own device memory.
 static __device__ __align__(256) int32_t g_phi_gaps_static[8 * (size_t)MVS_PHI_STATIC_MAX_PIXELS];
 
 // Device address of g_phi_gaps_static on the current device, looked up once
@@ -756,18 +860,27 @@ cudaError_t phi_static_scratch(int32_t** out) {
 cudaError_t launch_phi_hypotheses(int W, int H, const float* depth, const uint8_t* known, int n_fit, int inverse,
                                   float d_lo, float d_hi, float* hyp, uint8_t* valid, int32_t* scratch,
                                   cudaStream_t s) {
-    int maxl = W + H - 1;
-    dim3 grid(blocks_for(maxl, 128), 4);
-    k_line_gaps<<<grid, 128, 0, s>>>(W, H, known, scratch);
+    const LineMaps lm = line_maps(W, H, (uint32_t*)scratch);
+    const long long n = (long long)W * H;
+    const long long threads = std::max({32LL * H * lm.nwx, (long long)W * ((H + 31) / 32),
+                                        (long long)lm.nwp * (W + H - 1)});
+    k_line_bits<<<dim3(blocks_for(threads, 256), 4), 256, 0, s>>>(lm, known);
+    count_launch();
+    k_line_sums<<<dim3(blocks_for(std::max<long long>(H, (long long)W + H - 1) * ((std::max(lm.nwx, (H + 31) / 32) + 31) / 32),
+                                  256), 4), 256, 0, s>>>(lm);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    long long n = (long long)W * H;
-    k_line_fit<<<blocks_for(n, 128), 128, 0, s>>>(W, H, depth, known, scratch, n_fit, inverse, d_lo, d_hi, hyp,
-                                                  valid);
+    if (n_fit <= 8)
+        k_line_fit<8><<<blocks_for(4 * n, 256), 256, 0, s>>>(lm, depth, known, n_fit, inverse, d_lo, d_hi, hyp, valid);
+    else
+        k_line_fit<32><<<blocks_for(4 * n, 256), 256, 0, s>>>(lm, depth, known, n_fit, inverse, d_lo, d_hi, hyp, valid);
     count_launch();
     return cudaGetLastError();
 }
+
+// scratch of launch_phi_hypotheses, in 32-bit words (at most 8 per pixel)
+size_t phi_line_words(int W, int H) { return line_map_words(W, H); }
 
 #define MVS_DISPATCH(n, CALL)                       \
     do {                                            \
@@ -784,11 +897,11 @@ cudaError_t launch_phi_hypotheses(int W, int H, const float* depth, const uint8_
         else { CALL(32, 16); }                      \
     } while (0)
 
-cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t* valid, float* hcost,
+cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t* valid, float* hcost, int step,
                             cudaStream_t s) {
-    long long npix = (long long)rc.W * rc.H;
+    long long npix = (long long)((rc.W + step - 1) / step) * ((rc.H + step - 1) / step);
     const size_t smem = smem_block_bytes(rc.n_src, kWarps);
-#define CALL(G, S) k_phi_cost<G, S><<<pm_grid_for((const void*)k_phi_cost<G, S>, (npix + kWarps - 1) / kWarps, smem, kBlock), kBlock, smem, s>>>(rc, hyp, valid, hcost)
+#define CALL(G, S) k_phi_cost<G, S><<<pm_grid_for((const void*)k_phi_cost<G, S>, (npix + kWarps - 1) / kWarps, smem, kBlock), kBlock, smem, s>>>(rc, hyp, valid, hcost, step)
     MVS_DISPATCH(rc.n, CALL);
 #undef CALL
     count_launch();
