@@ -942,15 +942,18 @@ mvs_status mvs_sparse_depth_range(mvs_ctx* c, int32_t ref, int64_t n_points, con
     const int W = V.cam.width, H = V.cam.height;
     const size_t np = (size_t)n_points, npix = (size_t)W * H;
     auto a16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
-    size_t bytes = 16 + a16(np * sizeof(float2)) + a16(np * sizeof(float));
+    const size_t n_cells = 2 * sparse_range_cells(W, H) + 1;
+    size_t bytes = 16 + 2 * a16(np * sizeof(float4)) + a16(np * sizeof(int)) + a16(n_cells * sizeof(int));
     if (mem == MVS_MEM_HOST) bytes += a16(np * 3 * 8) + a16(np * 8) + a16(np * 8) + a16(np * 2 * 8) + a16(npix * 8);
     cudaError_t e;
     char* q = (char*)scratch(c, 7, bytes, &e);
     CK(c, e);
     auto take = [&](size_t b) { char* r = q; q += a16(b); return (void*)r; };
     unsigned long long* total = (unsigned long long*)take(16);
-    float2* uv = (float2*)take(np * sizeof(float2));
-    float* dep = (float*)take(np * sizeof(float));
+    float4* feat = (float4*)take(np * sizeof(float4));
+    float4* binned = (float4*)take(np * sizeof(float4));
+    int* cell_of = (int*)take(np * sizeof(int));
+    unsigned* cells = (unsigned*)take(n_cells * sizeof(unsigned));
     const double* dX = points;
     const unsigned long long* dvis = (const unsigned long long*)vis;
     const double* drep = reproj;
@@ -974,7 +977,7 @@ mvs_status mvs_sparse_depth_range(mvs_ctx* c, int32_t ref, int64_t n_points, con
     }
     const double Rrow2[3] = {V.cam.R[6], V.cam.R[7], V.cam.R[8]};
     CK(c, launch_sparse_range(ref, (int)c->views.size(), Rrow2, V.cam.t[2], dX, dvis, drep, dobs, (long long)np,
-                              max_reproj, W, H, d_lo, d_hi, total, uv, dep, drange, c->stream));
+                              max_reproj, W, H, d_lo, d_hi, total, feat, binned, cell_of, cells, drange, c->stream));
     if (mem == MVS_MEM_HOST) {
         CK(c, cudaMemcpyAsync(range, drange, npix * 8, cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
