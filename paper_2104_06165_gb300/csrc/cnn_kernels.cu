@@ -285,20 +285,6 @@ __global__ void k_pool_fwd_v(const uint4* __restrict__ in, int W, int H, int C, 
     }
 }
 
-// decoder input: out (W x H, up_ch + C) = [nearest up-sampling of prev
-// (W/2 x H/2, up_ch) | skip (W x H, C)], copies of 16-byte vectors
-__global__ void k_concat_up(const uint4* __restrict__ prev, int up_ch, const uint4* __restrict__ skip, int C, int W,
-                            int H, uint4* __restrict__ out) {
-    const int uv = up_ch / 8, sv = C / 8, ov = uv + sv;
-    const long long n = (long long)W * H * ov;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % ov);
-        const long long p = i / ov;
-        const int x = (int)(p % W), y = (int)(p / W);
-        out[i] = c < uv ? prev[((long long)(y / 2) * (W / 2) + x / 2) * uv + c] : skip[p * sv + (c - uv)];
-    }
-}
-
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                        long long n, float lr, float b1, float b2, float eps, float c1, float c2) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -381,20 +367,21 @@ __global__ void k_proposal_loss(const float* __restrict__ out, const float4* __r
     if ((threadIdx.x & 31) == 0 && lsum != 0.0f) atomicAdd(loss_sum, lsum);
 }
 
-// decode the head into K = 4 planes per pixel (n facing the camera, depth)
-__global__ void k_decode_proposals(const float* __restrict__ out, long long npix, int W, HeadConst hc, Mat3 Kinv,
+// decode the head into K = 4 planes per pixel (n facing the camera, depth),
+// one proposal per thread (one 16-byte load and store)
+__global__ void k_decode_proposals(const float4* __restrict__ out, long long npix, int W, HeadConst hc, Mat3 Kinv,
                                    float4* __restrict__ props) {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= npix) return;
-    int x = (int)(i % W), y = (int)(i / W);
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t >= 4 * npix) return;
+    const int i = (int)(t >> 2), y = i / W, x = i - y * W;   // at most 8192 x 8192 pixels
     float r0 = Kinv.m[0] * x + Kinv.m[1] * y + Kinv.m[2], r1 = Kinv.m[3] * x + Kinv.m[4] * y + Kinv.m[5];
     float r2 = Kinv.m[6] * x + Kinv.m[7] * y + Kinv.m[8];
-    for (int k = 0; k < 4; ++k) {
-        float rho, n[3], len, sig;
-        decode(out + 16 * i + 4 * k, hc, rho, n, len, sig);
-        if (n[0] * r0 + n[1] * r1 + n[2] * r2 > 0.0f) { n[0] = -n[0]; n[1] = -n[1]; n[2] = -n[2]; }
-        props[4 * i + k] = make_float4(n[0], n[1], n[2], 1.0f / rho);
-    }
+    const float4 v = out[t];
+    const float o[4] = {v.x, v.y, v.z, v.w};
+    float rho, n[3], len, sig;
+    decode(o, hc, rho, n, len, sig);
+    if (n[0] * r0 + n[1] * r1 + n[2] * r2 > 0.0f) { n[0] = -n[0]; n[1] = -n[1]; n[2] = -n[2]; }
+    props[t] = make_float4(n[0], n[1], n[2], 1.0f / rho);
 }
 
 // network input (16 channels, bf16): image / 255, normalised inverse depth,
@@ -486,7 +473,7 @@ constexpr unsigned kConvWaitLimit = 1u << 24;
 // One tensor-core convolution; `status` collects a timed-out wait.
 cudaError_t conv_launch(mvs_cnn* n, const bf16* in, int Cin, int W, int H, const bf16* wt, const float* bias,
                         int taps, int Cout, bool relu, bool out_f32, void* out, int out_ch, int out_off,
-                        cudaStream_t s);
+                        cudaStream_t s, const ConvExtra& extra = ConvExtra());
 
 cudaError_t wgrad_launch(const bf16* x, int Cin, const bf16* dy, int Cout, int W, int H, int taps, float* dw, float* db,
                          cudaStream_t s) {
@@ -536,8 +523,8 @@ cudaError_t refresh_bf16(mvs_cnn* n) {
 
 cudaError_t conv_launch(mvs_cnn* n, const bf16* in, int Cin, int W, int H, const bf16* wt, const float* bias,
                         int taps, int Cout, bool relu, bool out_f32, void* out, int out_ch, int out_off,
-                        cudaStream_t s) {
-    return conv_tc_launch(in, Cin, W, H, wt, bias, taps, Cout, relu, out_f32, out, out_ch, out_off, n->status, 0,
+                        cudaStream_t s, const ConvExtra& extra) {
+    return conv_tc_launch(in, Cin, W, H, wt, bias, taps, Cout, relu, out_f32, out, out_ch, out_off, extra, n->status, 0,
                           kConvWaitLimit, s);
 }
 
@@ -547,32 +534,42 @@ cudaError_t cnn_forward(mvs_cnn* n, int W, int H) {
     auto C = [&](int l) -> const Layer& { return n->L[l]; };
     int Ws[5], Hs[5];
     for (int l = 0; l < 5; ++l) { Ws[l] = W >> l; Hs[l] = H >> l; }
+    // decoder input of level l: c[l] = [up(d[l + 1] or e[4]) | e[l]], each part
+    // written by the convolution that computes it
+    auto cat_ch = [&](int l) { return C(D3 + (3 - l)).cin; };
     // encoder
     const bf16* in = n->x;
     for (int l = 0; l <= 4; ++l) {
         const Layer& L = C(E0 + l);
-        if (l > 0) {
-            k_pool_fwd_v<<<blocks((long long)Ws[l] * Hs[l] * C(E0 + l - 1).cout / 8), 256, 0, s>>>(
-                reinterpret_cast<const uint4*>(n->e[l - 1]), Ws[l - 1], Hs[l - 1], C(E0 + l - 1).cout,
-                reinterpret_cast<uint4*>(n->p[l - 1]));
-            count_launch();
-            in = n->p[l - 1];
+        ConvExtra x;
+        if (l < 4) {
+            x.skip = n->c[l];
+            x.skip_ch = cat_ch(l);
+            x.skip_off = cat_ch(l) - L.cout;
+            if (conv_tc_can_pool(9, L.cout, Ws[l], Hs[l])) x.pool = n->p[l];
+        } else {
+            x.up = n->c[3];
+            x.up_ch = cat_ch(3);
         }
-        CUK(conv_launch(n, in, L.cin, Ws[l], Hs[l], L.wt, L.b, 9, L.cout, true, false, n->e[l], L.cout, 0, s));
+        CUK(conv_launch(n, in, L.cin, Ws[l], Hs[l], L.wt, L.b, 9, L.cout, true, false, n->e[l], L.cout, 0, s, x));
+        if (l < 4) {
+            if (!x.pool) {
+                k_pool_fwd_v<<<blocks((long long)Ws[l + 1] * Hs[l + 1] * L.cout / 8), 256, 0, s>>>(
+                    reinterpret_cast<const uint4*>(n->e[l]), Ws[l], Hs[l], L.cout, reinterpret_cast<uint4*>(n->p[l]));
+                count_launch();
+            }
+            in = n->p[l];
+        }
     }
-    // decoder: level l = 3..0, c[l] = [up(prev) | e[l]]
-    const bf16* prev = n->e[4];
-    int prev_ch = C(E4).cout;
+    // decoder: level l = 3..0
     for (int l = 3; l >= 0; --l) {
         const Layer& L = C(D3 + (3 - l));
-        int ch = L.cin;
-        k_concat_up<<<blocks((long long)Ws[l] * Hs[l] * ch / 8), 256, 0, s>>>(
-            reinterpret_cast<const uint4*>(prev), prev_ch, reinterpret_cast<const uint4*>(n->e[l]), C(E0 + l).cout,
-            Ws[l], Hs[l], reinterpret_cast<uint4*>(n->c[l]));
-        count_launch();
-        CUK(conv_launch(n, n->c[l], ch, Ws[l], Hs[l], L.wt, L.b, 9, L.cout, true, false, n->d[l], L.cout, 0, s));
-        prev = n->d[l];
-        prev_ch = L.cout;
+        ConvExtra x;
+        if (l > 0) {
+            x.up = n->c[l - 1];
+            x.up_ch = cat_ch(l - 1);
+        }
+        CUK(conv_launch(n, n->c[l], L.cin, Ws[l], Hs[l], L.wt, L.b, 9, L.cout, true, false, n->d[l], L.cout, 0, s, x));
     }
     const Layer& Hd = C(HEAD);
     CUK(conv_launch(n, n->d[0], Hd.cin, W, H, Hd.wt, Hd.b, 1, Hd.cout, false, true, n->y, Hd.cout, 0, s));
@@ -667,7 +664,8 @@ cudaError_t cnn_propose(mvs_cnn* n, const uint8_t* img, const float4* plane, con
     if (e == cudaSuccess) {
         Mat3 K;
         for (int i = 0; i < 9; ++i) K.m[i] = (float)Kinv[i];
-        k_decode_proposals<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(n->y, np, W, n->hc, K, props);
+        k_decode_proposals<<<(unsigned)((4 * np + 255) / 256), 256, 0, s>>>(reinterpret_cast<const float4*>(n->y), np, W,
+                                                                           n->hc, K, props);
         count_launch();
         e = cudaGetLastError();
     }
@@ -913,7 +911,7 @@ mvs_status mvs_cnn_test_timeout(mvs_cnn* n) {
     // one 16 x 16 convolution of the input buffer whose first wait targets a
     // barrier that nothing completes, with a wait limit of about 0.1 ms
     CNK(n, conv_tc_launch(n->x, 16, 16, 16, n->L[E0].wt, n->L[E0].b, 9, n->L[E0].cout, true, false, n->e[0],
-                          n->L[E0].cout, 0, n->status, 1, 1500u, n->stream));
+                          n->L[E0].cout, 0, ConvExtra(), n->status, 1, 1500u, n->stream));
     CNK(n, cudaStreamSynchronize(n->stream));
     return check_status(n);
 }
