@@ -766,24 +766,25 @@ mvs_status mvs_fuse(mvs_ctx* c, int32_t n_views, const int32_t* views, const uin
     }
     CK(c, cudaSetDevice(c->device));
     // scratch slot 6, every region starting on a 16-byte boundary: per view
-    // the claim and alive arrays (and a device copy of a host keep mask),
+    // the claim and depth arrays (and a device copy of a host keep mask),
     // then block counts, block offsets, the running total and the views
     auto a16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
     const bool copy_keep = mem == MVS_MEM_HOST && keep_masks;
     size_t bytes = 0, max_blocks = 1;
     for (int a = 0; a < n_views; ++a) {
         const size_t np = (size_t)c->views[views[a]].cam.width * c->views[views[a]].cam.height;
-        bytes += a16(np * sizeof(int)) + a16(np) * (copy_keep ? 2 : 1);
+        bytes += a16(np * sizeof(int)) + a16(np * sizeof(float)) + (copy_keep ? a16(np) : 0);
         max_blocks = std::max(max_blocks, (np + 255) / 256);
     }
-    bytes += a16(max_blocks * sizeof(int)) + a16(max_blocks * sizeof(long long)) + 16 +
+    const size_t hits_bytes = max_blocks * 256 * sizeof(uint32_t);   // of the view being merged
+    bytes += hits_bytes + a16(max_blocks * sizeof(int)) + a16(max_blocks * sizeof(long long)) + 16 +
              a16((size_t)n_views * sizeof(FuseView));
     cudaError_t e;
     char* buf = (char*)scratch(c, 6, bytes, &e);
     CK(c, e);
     std::vector<FuseView> fv(n_views);
-    std::vector<const uint8_t*> keep_d(n_views, nullptr);
-    char* q = buf;
+    uint32_t* hits = (uint32_t*)buf;
+    char* q = buf + hits_bytes;
     for (int a = 0; a < n_views; ++a) {
         const ViewData& V = c->views[views[a]];
         const size_t np = (size_t)V.cam.width * V.cam.height;
@@ -798,16 +799,18 @@ mvs_status mvs_fuse(mvs_ctx* c, int32_t n_views, const int32_t* views, const uin
         f.plane = V.plane;
         f.claim = (int*)q;
         q += a16(np * sizeof(int));
-        f.alive = (uint8_t*)q;
-        q += a16(np);
+        f.depth = (float*)q;
+        q += a16(np * sizeof(float));
+        f.keep = nullptr;
+        f.hits = hits;
         if (copy_keep) {
             if (keep_masks[a]) {
                 CK(c, cudaMemcpyAsync(q, keep_masks[a], np, cudaMemcpyHostToDevice, c->stream));
-                keep_d[a] = (const uint8_t*)q;
+                f.keep = (const uint8_t*)q;
             }
             q += a16(np);
         } else if (keep_masks) {
-            keep_d[a] = keep_masks[a];
+            f.keep = keep_masks[a];
         }
     }
     int* block_count = (int*)q;
@@ -839,7 +842,7 @@ mvs_status mvs_fuse(mvs_ctx* c, int32_t n_views, const int32_t* views, const uin
             off += (size_t)fv[a].W * fv[a].H;
         }
     }
-    CK(c, launch_fuse(fv.data(), dev_views, n_views, keep_masks ? keep_d.data() : nullptr, rel_tol, block_count,
+    CK(c, launch_fuse(fv.data(), dev_views, n_views, rel_tol, block_count,
                       block_off, total, pts_d, src_d, capacity, c->stream));
     long long tot = 0;
     CK(c, cudaMemcpyAsync(&tot, total, sizeof tot, cudaMemcpyDeviceToHost, c->stream));

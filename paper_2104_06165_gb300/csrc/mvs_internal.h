@@ -183,13 +183,16 @@ struct FuseView {
     int W, H;
     int index;                   // context view index (reported with each point)
     const float4* plane;         // depth map (depth in .w, 0 = none)
-    uint8_t* alive;              // W*H: 1 = still present
+    const uint8_t* keep;         // W*H or NULL: pixels that take part
+    float* depth;                // W*H: depth of the pixels still present, else 0
+    uint32_t* hits;              // W*H: later views the pixel claimed from (one buffer for all views)
     int* claim;                  // W*H: lowest claiming pixel of the view being fused
     long long* owner;            // W*H or NULL: index of the point the pixel went into, -1 if absent
 };
-cudaError_t launch_fuse(const FuseView* host_views, FuseView* dev_views, int n, const uint8_t* const* keep, float tol,
-                        int* block_count, long long* block_off, long long* total, float4* points, int2* src,
-                        long long cap, cudaStream_t s);
+// (total: two words, the running total and a counter)
+cudaError_t launch_fuse(const FuseView* host_views, FuseView* dev_views, int n, float tol, int* block_count,
+                        long long* block_off, long long* total, float4* points, int2* src, long long cap,
+                        cudaStream_t s);
 
 // neighbouring-image selection (select_kernels.cu): at most 64 views (one
 // visibility bit per view in a 64-bit mask per sparse point)
