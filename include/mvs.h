@@ -173,6 +173,11 @@ const char* mvs_last_error(const mvs_ctx* ctx);
  *   out: caller buffers of the reference's size; with MVS_INIT_GIVEN* they
  *   also carry the starting state.  The result is kept in the context for
  *   mvs_geo_filter / mvs_plane_infer.
+ *   The context keeps a workspace for its largest view: 20 bytes per pixel
+ *   and, when the call initialises or runs at least two iterations, each
+ *   pixel's reference window (8 bytes per sample slot and 64 more, 1088 bytes
+ *   for 11 x 11 samples) if all of them take at most 16 GiB and fit the device;
+ *   otherwise the windows are rebuilt at every visit, with the same results.
  * Errors: MVS_EINVAL (bad index, duplicate or self source, n_src outside
  *   1..32, window outside 2..22 samples, d_lo >= d_hi, NULL buffers),
  *   MVS_EUNSUPPORTED (precision other than 0 or 1), MVS_ENOMEM, MVS_ECUDA. */
@@ -323,7 +328,9 @@ mvs_status mvs_sparse_depth_range(mvs_ctx* ctx, int32_t ref, int64_t n_points, c
  *   context's copy of the view is updated.  pm gives the window / ZNCC
  *   parameters for the hypothesis costs.
  * Errors: MVS_ESTATE if the view has no depth map, MVS_EINVAL (also for an
- *   unknown selection), MVS_ECUDA. */
+ *   unknown selection), MVS_ECUDA, MVS_ETIMEOUT once a bounded wait of the
+ *   message passing ran out (with host buffers by this call, else by the next
+ *   one; mvs_phi_mrf likewise). */
 mvs_status mvs_plane_infer(mvs_ctx* ctx, int32_t ref, const int32_t* srcs, int32_t n_src,
                            const mvs_pm_params* pm, const mvs_phi_params* phi, const uint8_t* keep_mask,
                            mvs_depth_map* inout);
@@ -368,7 +375,7 @@ mvs_status mvs_phi_select_min_cost(mvs_ctx* ctx, int32_t ref, const uint8_t* kno
  *   every byte of the device, or a latency-bound pipeline that cannot afford
  *   the device-wide synchronisation cudaMalloc / cudaFree imply.  This entry
  *   point computes exactly what mvs_phi_hypotheses computes but keeps its
- *   line-gap scratch in a fixed array compiled into the library
+ *   line-map scratch in a fixed array compiled into the library
  *   (MVS_PHI_STATIC_MAX_PIXELS pixels x 32 bytes = 8 MiB per device, held by
  *   every device that loads the library until the process exits), so it
  *   calls no cudaMalloc, cudaFree or allocating library routine.
