@@ -945,7 +945,7 @@ mvs_status mvs_sparse_depth_range(mvs_ctx* c, int32_t ref, int64_t n_points, con
     const int W = V.cam.width, H = V.cam.height;
     const size_t np = (size_t)n_points, npix = (size_t)W * H;
     auto a16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
-    const size_t n_cells = 2 * sparse_range_cells(W, H) + 1;
+    const size_t n_cells = 2 * sparse_range_cells(W, H, (long long)np) + 1;
     size_t bytes = 16 + 2 * a16(np * sizeof(float4)) + a16(np * sizeof(int)) + a16(n_cells * sizeof(int));
     if (mem == MVS_MEM_HOST) bytes += a16(np * 3 * 8) + a16(np * 8) + a16(np * 8) + a16(np * 2 * 8) + a16(npix * 8);
     cudaError_t e;

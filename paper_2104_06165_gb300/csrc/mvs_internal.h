@@ -211,7 +211,7 @@ cudaError_t launch_sparse_range(int ref, int n_views, const double Rrow2[3], dou
                                 long long n_pts, double max_reproj, int W, int H, float d_lo, float d_hi,
                                 unsigned long long* total, float4* feat, float4* binned, int* cell_of, unsigned* cells,
                                 float2* range, cudaStream_t s);
-size_t sparse_range_cells(int W, int H);   // `cells` holds twice as many words and one more
+size_t sparse_range_cells(int W, int H, long long n_pts);   // `cells` holds twice as many words and one more
 
 // learned proposals (cnn_kernels.cu)
 struct mvs_cnn;

@@ -133,14 +133,14 @@ cudaError_t launch_select_neighbors(const NbrView* dev_views, int n, const doubl
 // precision, each operation rounded on its own, the first feature winning a
 // tie.
 //
-// The features are binned into cells of kCell px and a warp looks at the cells
-// in rings around its pixels until no farther feature can matter, instead of
-// every tile scanning every point: what is left is about the features nearby
-// (3072 x 2048, 20 k points: 0.48 ms for the whole call against 6.1 ms).
+// With many tiles and points the features are binned into cells and a warp
+// looks at the cells in rings around its pixels until no farther feature can
+// matter, so that what is left is about the features nearby (3072 x 2048, 20 k
+// points: 0.39 ms for the whole call; 3.8 ms with every tile scanning every
+// point, which is the faster way for the small calls, see all_features).
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int kCell = 32;
 // pixels of a block: 16 x 16, a warp covers 16 x 2 (inside one cell)
 constexpr int kRangeTile = 16;
 
@@ -157,7 +157,7 @@ __global__ void k_sparse_features(const double* __restrict__ X, const unsigned l
                                   const double* __restrict__ reproj, const double* __restrict__ obs, long long n_pts,
                                   unsigned long long views_mask, const unsigned long long* __restrict__ total,
                                   int ref, double R6, double R7, double R8, double t2, double max_reproj,
-                                  int ncx, int ncy, float4* __restrict__ feat, int* __restrict__ cell_of,
+                                  int cell, int ncx, int ncy, float4* __restrict__ feat, int* __restrict__ cell_of,
                                   unsigned* __restrict__ cell_n) {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (p >= n_pts) return;
@@ -168,17 +168,20 @@ __global__ void k_sparse_features(const double* __restrict__ X, const unsigned l
     double z = __dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(R6, X[3 * p]), __dmul_rn(R7, X[3 * p + 1])),
                                    __dmul_rn(R8, X[3 * p + 2])),
                          t2);
-    const float u = (float)obs[2 * p], v = (float)obs[2 * p + 1];
+    const float u = (float)obs[2 * p], v = (float)obs[2 * p + 1], zf = (float)z;
+    // a feature without a depth is none
+    const bool feature = keep && isfinite(u) && isfinite(v) && zf == zf;
+    feat[p] = make_float4(u, v, feature ? zf : __int_as_float(0x7fc00000), __uint_as_float((uint32_t)p));
+    if (!cell_of) return;
     int c = -1;
-    if (keep && isfinite(u) && isfinite(v)) {
+    if (feature) {
         // features outside the image go to the cells at its edge
-        const int cx = (int)fminf(fmaxf(u * (1.0f / kCell), 0.0f), (float)(ncx - 1));
-        const int cy = (int)fminf(fmaxf(v * (1.0f / kCell), 0.0f), (float)(ncy - 1));
+        const int cx = (int)fminf(fmaxf(u, 0.0f), (float)(ncx * cell - 1)) / cell;
+        const int cy = (int)fminf(fmaxf(v, 0.0f), (float)(ncy * cell - 1)) / cell;
         c = cy * ncx + cx;
         atomicAdd(cell_n + c, 1u);
     }
     cell_of[p] = c;
-    feat[p] = make_float4(u, v, (float)z, __uint_as_float((uint32_t)p));
 }
 
 // exclusive scan of the cell counts (one block), counts cleared for the filling
@@ -215,13 +218,25 @@ __global__ void k_sparse_fill(const float4* __restrict__ feat, const int* __rest
     if (c >= 0) binned[cell_start[c] + atomicAdd(cell_n + c, 1u)] = feat[p];
 }
 
+__device__ __forceinline__ float2 span(const float best[4], const float bd[4], float d_lo, float d_hi) {
+    float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (best[q] < INFINITY) {
+            lo = bd[q] < lo ? bd[q] : lo;
+            hi = bd[q] > hi ? bd[q] : hi;
+        }
+    const float nan = __int_as_float(0x7fc00000);
+    return lo <= hi ? make_float2(fminf(fmaxf(lo, d_lo), d_hi), fminf(fmaxf(hi, d_lo), d_hi)) : make_float2(nan, nan);
+}
+
 __global__ void __launch_bounds__(kRangeTile * kRangeTile) k_sparse_range(
-    const float4* __restrict__ binned, const unsigned* __restrict__ cell_start, int ncx, int ncy, int W, int H, float d_lo,
-    float d_hi, float2* __restrict__ range) {
+    const float4* __restrict__ binned, const unsigned* __restrict__ cell_start, int cell, int ncx, int ncy, int W, int H,
+    float d_lo, float d_hi, float2* __restrict__ range) {
     const int x = blockIdx.x * kRangeTile + (threadIdx.x % kRangeTile);
     const int y = blockIdx.y * kRangeTile + (threadIdx.x / kRangeTile);
     const float r = __fdiv_rn((float)W, 10.0f), r2 = __fmul_rn(r, r);
-    const int cx = blockIdx.x * kRangeTile / kCell, cy = blockIdx.y * kRangeTile / kCell;
+    const int cx = blockIdx.x * kRangeTile / cell, cy = blockIdx.y * kRangeTile / cell;
     // quadrants: 0 right / lower, 1 left / lower, 2 left / upper, 3 right / upper
     float best[4] = {INFINITY, INFINITY, INFINITY, INFINITY}, bd[4] = {0.f, 0.f, 0.f, 0.f};
     uint32_t bi[4] = {0u, 0u, 0u, 0u};
@@ -262,10 +277,10 @@ __global__ void __launch_bounds__(kRangeTile * kRangeTile) k_sparse_range(
         // distance of the features not seen yet: beyond the square of cells
         // looked at (to infinity where it has reached the edge of the grid);
         // 0.01 px covers the rounding of the compared distances
-        const float el = cx - k > 0 ? fx - (float)((cx - k) * kCell) : INFINITY;
-        const float er = cx + k < ncx - 1 ? (float)((cx + k + 1) * kCell) - fx : INFINITY;
-        const float eu = cy - k > 0 ? fy - (float)((cy - k) * kCell) : INFINITY;
-        const float ed = cy + k < ncy - 1 ? (float)((cy + k + 1) * kCell) - fy : INFINITY;
+        const float el = cx - k > 0 ? fx - (float)((cx - k) * cell) : INFINITY;
+        const float er = cx + k < ncx - 1 ? (float)((cx + k + 1) * cell) - fx : INFINITY;
+        const float eu = cy - k > 0 ? fy - (float)((cy - k) * cell) : INFINITY;
+        const float ed = cy + k < ncy - 1 ? (float)((cy + k + 1) * cell) - fy : INFINITY;
         bool done = true;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -274,45 +289,137 @@ __global__ void __launch_bounds__(kRangeTile * kRangeTile) k_sparse_range(
         }
         if (__all_sync(0xffffffffu, done || x >= W || y >= H)) break;
     }
-    if (x >= W || y >= H) return;
-    float lo = INFINITY, hi = -INFINITY;
-    for (int q = 0; q < 4; ++q)
-        if (best[q] < INFINITY) {
-            lo = bd[q] < lo ? bd[q] : lo;
-            hi = bd[q] > hi ? bd[q] : hi;
+    if (x < W && y < H) range[(long long)y * W + x] = span(best, bd, d_lo, d_hi);
+}
+
+// Every feature against every tile: 1024 features per step are compacted to
+// those within the radius of the tile, in the order of the points, so a
+// strict comparison keeps the first of a tie.
+__global__ void __launch_bounds__(kRangeTile * kRangeTile) k_sparse_range_all(
+    const float4* __restrict__ feat, long long n_pts, int W, int H, float d_lo, float d_hi, float2* __restrict__ range) {
+    constexpr int NT = kRangeTile * kRangeTile, NW = NT / 32, U = 4;
+    __shared__ float2 s_uv[U * NT];
+    __shared__ float s_d[U * NT];
+    __shared__ int s_wc[U * NW];
+    const int x = blockIdx.x * kRangeTile + (threadIdx.x % kRangeTile);
+    const int y = blockIdx.y * kRangeTile + (threadIdx.x / kRangeTile);
+    const float r = __fdiv_rn((float)W, 10.0f), r2 = __fmul_rn(r, r);
+    const float bx0 = (float)(blockIdx.x * kRangeTile) - r, bx1 = (float)(blockIdx.x * kRangeTile + kRangeTile - 1) + r;
+    const float by0 = (float)(blockIdx.y * kRangeTile) - r, by1 = (float)(blockIdx.y * kRangeTile + kRangeTile - 1) + r;
+    float best[4] = {INFINITY, INFINITY, INFINITY, INFINITY}, bd[4] = {0.f, 0.f, 0.f, 0.f};
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (long long base = 0; base < n_pts; base += U * NT) {
+        float4 f[U];
+        unsigned m[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const long long p = base + i * NT + threadIdx.x;
+            f[i] = p < n_pts ? __ldg(feat + p) : make_float4(0.f, 0.f, __int_as_float(0x7fc00000), 0.f);
         }
-    const float nan = __int_as_float(0x7fc00000);
-    range[(long long)y * W + x] = lo <= hi ? make_float2(fminf(fmaxf(lo, d_lo), d_hi), fminf(fmaxf(hi, d_lo), d_hi))
-                                           : make_float2(nan, nan);
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            m[i] = __ballot_sync(0xffffffffu, f[i].z == f[i].z && f[i].x >= bx0 && f[i].x <= bx1 && f[i].y >= by0 &&
+                                                  f[i].y <= by1);
+            if (lane == 0) s_wc[i * NW + warp] = __popc(m[i]);
+        }
+        __syncthreads();
+        static_assert(U * NW == 32, "one count per lane");
+        int incl = s_wc[lane];
+        const int own = incl;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const int cnt = __shfl_sync(0xffffffffu, incl, 31);
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int off = __shfl_sync(0xffffffffu, incl - own, i * NW + warp) + __popc(m[i] & ((1u << lane) - 1u));
+            if ((m[i] >> lane) & 1u) {
+                s_uv[off] = make_float2(f[i].x, f[i].y);
+                s_d[off] = f[i].z;
+            }
+        }
+        __syncthreads();
+        for (int k = 0; k < cnt; ++k) {
+            const float dx = __fsub_rn(s_uv[k].x, (float)x), dy = __fsub_rn(s_uv[k].y, (float)y);
+            const float d2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
+            if (!(d2 < r2)) continue;
+            const int q = dx >= 0.0f ? (dy >= 0.0f ? 0 : 3) : (dy >= 0.0f ? 1 : 2);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (j == q && d2 < best[j]) {
+                    best[j] = d2;
+                    bd[j] = s_d[k];
+                }
+        }
+        if (base + U * NT < n_pts) __syncthreads();
+    }
+    if (x < W && y < H) range[(long long)y * W + x] = span(best, bd, d_lo, d_hi);
+}
+
+// Side of the cells: about 3 points to a cell, so that the rings end after one
+// or two steps at any density (a fixed side of 32 pixels has up to ten rings of
+// empty cells where the points are few); a multiple of the tile, no more than
+// the radius needs.
+int cell_side(int W, int H, long long n_pts) {
+    const double side = std::sqrt(3.25 * (double)W * H / (double)std::max(1LL, n_pts));
+    const int most = (W / 10 + kRangeTile) / kRangeTile;
+    return kRangeTile * std::max(1, std::min(most, (int)(side / kRangeTile + 0.5)));
+}
+
+// Where every tile looks at every feature.  Binning costs three launches and
+// the rings a chain of dependent reads, about 20 us more than the scan at the
+// smallest sizes; the scan grows with tiles x points.  Scan against cells,
+// microseconds of a call: 320 x 240 18 / 39 with 1 k points and 104 / 177 with
+// 20 k (one wave of tiles: the scan's latency, and cells of 16 pixels hold too
+// many points there), 640 x 480 43 / 54 with 2.5 k and 81 / 72 with 6 k,
+// 960 x 640 36 / 53 and 70 / 66 with 1 k and 2.5 k, 3072 x 2048 221 / 247 with
+// 1 k, 526 / 273 with 2.5 k and 3807 / 392 with 20 k.
+bool all_features(int W, int H, long long n_pts) {
+    const long long tiles = (long long)((W + kRangeTile - 1) / kRangeTile) * ((H + kRangeTile - 1) / kRangeTile);
+    return tiles <= 4 * 152 || n_pts <= 1000 || tiles * n_pts <= 5000000;
 }
 
 }  // namespace
 
-size_t sparse_range_cells(int W, int H) { return (size_t)((W + kCell - 1) / kCell) * ((H + kCell - 1) / kCell); }
+size_t sparse_range_cells(int W, int H, long long n_pts) {
+    if (all_features(W, H, n_pts)) return 0;
+    const int cell = cell_side(W, H, n_pts);
+    return (size_t)((W + cell - 1) / cell) * ((H + cell - 1) / cell);
+}
 
 cudaError_t launch_sparse_range(int ref, int n_views, const double Rrow2[3], double t2, const double* X,
                                 const unsigned long long* vis, const double* reproj, const double* obs,
                                 long long n_pts, double max_reproj, int W, int H, float d_lo, float d_hi,
                                 unsigned long long* total, float4* feat, float4* binned, int* cell_of, unsigned* cells,
                                 float2* range, cudaStream_t s) {
-    const int ncx = (W + kCell - 1) / kCell, ncy = (H + kCell - 1) / kCell, nc = ncx * ncy;
+    const bool all = all_features(W, H, n_pts);
+    const int cell = cell_side(W, H, n_pts), ncx = (W + cell - 1) / cell, ncy = (H + cell - 1) / cell, nc = ncx * ncy;
     unsigned *cell_n = cells, *cell_start = cells + nc;
     cudaError_t e = cudaMemsetAsync(total, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(cells, 0, (2 * (size_t)nc + 1) * sizeof(int), s)) != cudaSuccess) return e;
+    if (!all && (e = cudaMemsetAsync(cell_n, 0, (size_t)nc * sizeof(unsigned), s)) != cudaSuccess) return e;
     const unsigned long long views_mask = n_views >= 64 ? ~0ULL : ((1ULL << n_views) - 1ULL);
     if (n_pts > 0) {
         const unsigned nb = (unsigned)std::min<long long>((n_pts + 255) / 256, 152LL * 8), np = (unsigned)((n_pts + 255) / 256);
         k_sparse_count<<<nb, 256, 0, s>>>(vis, n_pts, views_mask, total);
         k_sparse_features<<<np, 256, 0, s>>>(X, vis, reproj, obs, n_pts, views_mask, total, ref, Rrow2[0], Rrow2[1],
-                                             Rrow2[2], t2, max_reproj, ncx, ncy, feat, cell_of, cell_n);
-        k_sparse_scan<<<1, 1024, 0, s>>>(cell_n, cell_start, nc);
-        k_sparse_fill<<<np, 256, 0, s>>>(feat, cell_of, n_pts, cell_start, cell_n, binned);
-        count_launch(4);
+                                             Rrow2[2], t2, max_reproj, cell, ncx, ncy, feat, all ? nullptr : cell_of,
+                                             cell_n);
+        count_launch(2);
+        if (!all) {
+            k_sparse_scan<<<1, 1024, 0, s>>>(cell_n, cell_start, nc);
+            k_sparse_fill<<<np, 256, 0, s>>>(feat, cell_of, n_pts, cell_start, cell_n, binned);
+            count_launch(2);
+        }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     dim3 grid((W + kRangeTile - 1) / kRangeTile, (H + kRangeTile - 1) / kRangeTile);
-    k_sparse_range<<<grid, kRangeTile * kRangeTile, 0, s>>>(binned, cell_start, ncx, ncy, W, H, d_lo, d_hi, range);
+    if (all)
+        k_sparse_range_all<<<grid, kRangeTile * kRangeTile, 0, s>>>(feat, n_pts, W, H, d_lo, d_hi, range);
+    else
+        k_sparse_range<<<grid, kRangeTile * kRangeTile, 0, s>>>(binned, cell_start, cell, ncx, ncy, W, H, d_lo, d_hi, range);
     count_launch();
     return cudaGetLastError();
 }
