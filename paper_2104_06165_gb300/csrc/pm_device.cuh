@@ -41,25 +41,6 @@ __device__ __forceinline__ float add_f16_f32(__half h, float c) {
     return d;
 }
 
-// Two floats in a register pair; each half of a packed operation rounds like
-// the scalar one.
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 pack_f2(float x, float y) {
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ void unpack_f2(F2 a, float& x, float& y) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
-}
-__device__ __forceinline__ F2 fma_f2(F2 a, F2 b, F2 c) {
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-
 // Philox4x64-10 (Salmon et al., SC'11).
 __device__ __forceinline__ void philox4x64(unsigned long long c[4], unsigned long long k0,
                                            unsigned long long k1) {
@@ -516,13 +497,13 @@ __device__ __forceinline__ Cand make_cand(const RefConst& rc, const PixWin<S>& p
 // (ax, ay) of tex_sample and (hypothesis | view << 8 | fp16 coefficient a of
 // the texel at the anchor << 16).
 struct __align__(16) PairSm {
-    float j0x, j0y, j1x, j1y;
-    float nx, ny, mx, my;
-    float h0z, h1z, pz;
+    float j0x, j0y, h0z, j1x;
+    float j1y, h1z, nx, ny;
+    float pz, mx, my;
     int cj;
 };
 
-static_assert(sizeof(PairSm) == 48 && offsetof(PairSm, nx) == 16 && offsetof(PairSm, h0z) == 32 &&
+static_assert(sizeof(PairSm) == 48 && offsetof(PairSm, j1y) == 16 && offsetof(PairSm, pz) == 32 &&
                   offsetof(PairSm, cj) == 44,
               "eval_batch reads and writes PairSm as 128-bit words");
 
@@ -559,7 +540,7 @@ __device__ __forceinline__ bool same_plane(const float4& a, const float4& b) {
 // The anchored homography of one listed pair (PairSm words 0..2 without the
 // (hypothesis, view) word).
 struct PairGeo {
-    float j0x, j0y, j1x, j1y, nx, ny, mx, my, h0z, h1z, pz;
+    float j0x, j0y, h0z, j1x, j1y, h1z, nx, ny, pz, mx, my;
 };
 
 // One pass over a group's window samples of a listed pair (S slots per lane).
@@ -577,9 +558,7 @@ struct PairGeo {
 //   CENTRED = false: sa, sb, se += sum w d, sum w d^2, sum w r' d over the
 //     lane's samples, d = s - c0 (nc0 = -c0);
 //   CENTRED = true: sa += sum w (d - mean_d)^2.
-// The gathers run in chunks of up to 9 slots (registers).  x and y of a sample
-// go through packed operations (half the instructions of these steps; learned
-// run in mixed precision 24.9 -> 24.1 ms, FP32 maps the same within 1 %).
+// The gathers run in chunks of up to 9 slots (registers).
 template <int G, int S, bool CENTRED, int CH = (S <= 9 ? S : (S + 1) / 2)>
 __device__ __forceinline__ void window_pass(const PixWin<S>& pw, int grp,
                                             const uint2* __restrict__ tex, uint32_t pitch, uint32_t last,
@@ -594,15 +573,13 @@ __device__ __forceinline__ void window_pass(const PixWin<S>& pw, int grp,
             const int k = k0 + kk;
             if (k < S) {
                 const float2 o = unpack_offset(pw.o2[k]);
-                const F2 j0 = pack_f2(g.j0x, g.j0y), j1 = pack_f2(g.j1x, g.j1y), nn = pack_f2(g.nx, g.ny);
-                const F2 mm = pack_f2(g.mx, g.my), neg = pack_f2(-1.0f, -1.0f);
-                const F2 XY = fma_f2(pack_f2(o.x, o.x), j0, fma_f2(pack_f2(o.y, o.y), j1, nn));
+                const float X = fmaf(o.x, g.j0x, fmaf(o.y, g.j1x, g.nx));
+                const float Y = fmaf(o.x, g.j0y, fmaf(o.y, g.j1y, g.ny));
                 const float Z = fmaf(o.x, g.h0z, fmaf(o.y, g.h1z, g.pz));
                 const float iz = rcp_approx(Z);
-                const F2 izz = pack_f2(iz, iz), txy = fma_f2(XY, izz, mm);
-                float tx, ty;
-                unpack_f2(txy, tx, ty);
-                unpack_f2(fma_f2(XY, izz, fma_f2(txy, neg, mm)), Us[kk], Vs[kk]);
+                const float tx = fmaf(X, iz, g.mx), ty = fmaf(Y, iz, g.my);
+                Us[kk] = fmaf(X, iz, g.mx - tx);
+                Vs[kk] = fmaf(Y, iz, g.my - ty);
                 // (j + 1) pitch + (i + 1) modulo 2^32 (tex_fold)
                 const uint32_t idx = (uint32_t)__float_as_int(ty) * pitch + (uint32_t)__float_as_int(tx);
                 tq[kk] = __ldg(tex + min(idx, last));
@@ -657,15 +634,13 @@ __device__ __forceinline__ void window_pass_h2(const PixWin<S>& pw, const uint2*
             const int k = k0 + kk;
             if (k < S) {
                 const float2 o = unpack_offset(pw.o2[k]);
-                const F2 j0 = pack_f2(g.j0x, g.j0y), j1 = pack_f2(g.j1x, g.j1y), nn = pack_f2(g.nx, g.ny);
-                const F2 mm = pack_f2(g.mx, g.my), neg = pack_f2(-1.0f, -1.0f);
-                const F2 XY = fma_f2(pack_f2(o.x, o.x), j0, fma_f2(pack_f2(o.y, o.y), j1, nn));
+                const float X = fmaf(o.x, g.j0x, fmaf(o.y, g.j1x, g.nx));
+                const float Y = fmaf(o.x, g.j0y, fmaf(o.y, g.j1y, g.ny));
                 const float Z = fmaf(o.x, g.h0z, fmaf(o.y, g.h1z, g.pz));
                 const float iz = rcp_approx(Z);
-                const F2 izz = pack_f2(iz, iz), txy = fma_f2(XY, izz, mm);
-                float tx, ty;
-                unpack_f2(txy, tx, ty);
-                unpack_f2(fma_f2(XY, izz, fma_f2(txy, neg, mm)), Us[kk], Vs[kk]);
+                const float tx = fmaf(X, iz, g.mx), ty = fmaf(Y, iz, g.my);
+                Us[kk] = fmaf(X, iz, g.mx - tx);
+                Vs[kk] = fmaf(Y, iz, g.my - ty);
                 const uint32_t idx = (uint32_t)__float_as_int(ty) * pitch + (uint32_t)__float_as_int(tx);
                 tq[kk] = __ldg(tex + min(idx, last));
             }
@@ -810,7 +785,8 @@ __device__ __forceinline__ float eval_batch(const RefConst& rc, const ViewSm* __
             float4* qw = reinterpret_cast<float4*>(pairs + count + __popc(m & ((1u << lane) - 1u)));
             // derivatives per sample step (the offsets are in steps)
             const float st = rc.step;
-            qw[0] = make_float4(j0x * st, j0y * st, j1x * st, j1y * st);
+            qw[0] = make_float4(j0x * st, j0y * st, h0z * st, j1x * st);
+            qw[1] = make_float4(j1y * st, h1z * st, nx, ny);
             // magic numbers with the anchor, the texture's guard texel and the
             // index fold (tex_fold): bits(ty) pitch + bits(tx) = texel index
             const float mx = kMagic2 + (ax + w1.x), my = kMagic2 + (ay + w1.y);
@@ -820,8 +796,7 @@ __device__ __forceinline__ float eval_batch(const RefConst& rc, const ViewSm* __
             const uint2* tex = reinterpret_cast<const uint2*>(((unsigned long long)v0.y << 32) | v0.x);
             const uint32_t ia = (uint32_t)__float_as_int(my) * v0.z + (uint32_t)__float_as_int(mx);
             const uint32_t a16 = __ldg(reinterpret_cast<const unsigned short*>(tex + min(ia, v0.w)));
-            qw[1] = make_float4(nx, ny, mx, my);
-            qw[2] = make_float4(h0z * st, h1z * st, pz, __uint_as_float((uint32_t)c | ((uint32_t)j << 8) | (a16 << 16)));
+            qw[2] = make_float4(pz, mx, my, __uint_as_float((uint32_t)c | ((uint32_t)j << 8) | (a16 << 16)));
         } else if (act) {
             tab[c * V + j] = 0.0f;   // view excluded for this hypothesis
         }
