@@ -12,6 +12,7 @@
 
 #include "../../include/mvs.h"
 #include "mvs_internal.h"
+#include "workspace.h"
 
 namespace {
 
@@ -56,7 +57,8 @@ struct mvs_ctx {
     cudaStream_t stream = nullptr;
     std::vector<ViewData> views;
     std::string err;
-    Scratch scratch[9];
+    Scratch scratch[8];
+    PhaseWorkspace work;                   // of the checkerboard phases, shared by the views
     // measurement hooks
     bool prof = false;
     std::vector<cudaEvent_t> ev;
@@ -266,30 +268,44 @@ mvs_status ensure_map(mvs_ctx* c, int32_t v) {
     return MVS_OK;
 }
 
+// device memory of a context's workspace
+struct CtxMemory {
+    mvs_ctx* c;
+    cudaError_t err = cudaSuccess;   // of the last get
+    void* get(size_t bytes) {
+        void* p = nullptr;
+        err = cudaMalloc(&p, bytes);
+        if (err == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
+    }
+    bool full() const { return err == cudaErrorMemoryAllocation; }
+    void put(void* p) {
+        cudaStreamSynchronize(c->stream);
+        cudaFree(p);
+    }
+};
+
 // The phases' workspace, one per context (its views run one after another):
-// the refinement perturbations of an iteration (20 bytes per pixel), then, when
+// the refinement perturbations of an iteration (20 bytes per pixel) and, when
 // the call visits every pixel often enough to pay for storing the windows (an
 // initialisation, which builds them anyway, or at least two iterations) and
-// they take at most kWindowBytes, the stored windows; otherwise the phases
-// rebuild each window, with the same results.
-constexpr size_t kWindowBytes = (size_t)16 << 30;
-cudaError_t use_workspace(mvs_ctx* c, RefConst& rc, size_t max_pixels, const mvs_pm_params* p, int phases) {
+// they fit, the stored windows; otherwise the phases rebuild each window, with
+// the same results.  One choice for all n views of a call, of at most
+// max_pixels pixels each and with the same window.
+cudaError_t use_workspace(mvs_ctx* c, RefConst* rcs, int n, size_t max_pixels, const mvs_pm_params* p, int phases) {
     if (phases == 0) return cudaSuccess;
     const bool init = p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE;
-    const size_t draws = (max_pixels * 20 + 255) & ~(size_t)255;
-    size_t windows = phases >= (init ? 1 : 4) ? max_pixels * pm_window_bytes(rc) : 0;
-    if (windows > kWindowBytes) windows = 0;
-    cudaError_t e;
-    char* b = (char*)scratch(c, 8, draws + windows, &e);
-    if (e != cudaSuccess && windows) {   // no room for the windows
-        cudaGetLastError();
-        windows = 0;
-        b = (char*)scratch(c, 8, draws, &e);
+    const size_t windows = phases >= (init ? 1 : 4) ? max_pixels * pm_window_bytes(rcs[0]) : 0;
+    CtxMemory mem{c};
+    bool stored = false;
+    if (!ws_reserve(c->work, max_pixels * 20, windows, &stored, mem)) return mem.err;
+    char* const draws = (char*)c->work.draws.p;
+    for (int r = 0; r < n; ++r) {
+        rcs[r].draw4 = (float4*)draws;
+        rcs[r].draw1 = (float*)(draws + max_pixels * 16);
+        rcs[r].win = stored ? (float*)c->work.windows.p : nullptr;
     }
-    if (e != cudaSuccess) return e;
-    rc.draw4 = (float4*)b;
-    rc.draw1 = (float*)(b + max_pixels * 16);
-    rc.win = windows ? (float*)(b + draws) : nullptr;
     return cudaSuccess;
 }
 
@@ -375,6 +391,8 @@ void mvs_destroy(mvs_ctx* c) {
         cudaFree(V.gen);
     }
     for (auto& s : c->scratch) cudaFree(s.p);
+    cudaFree(c->work.draws.p);
+    cudaFree(c->work.windows.p);
     for (auto e : c->ev) cudaEventDestroy(e);
     cudaFree(c->evals);
     cudaFreeHost(c->wait_status);
@@ -414,7 +432,7 @@ mvs_status mvs_patchmatch(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t 
     RefConst rc;
     make_refconst(c, ref, srcs, n_src, p, rc);
     const bool init = p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE;
-    CK(c, use_workspace(c, rc, n, p, pend - p->phase_begin));
+    CK(c, use_workspace(c, &rc, 1, n, p, pend - p->phase_begin));
     if (rc.win && !init) CK(c, launch_windows(rc, c->stream));
     if (init) {
         CK(c, launch_init(rc, c->stream));
@@ -485,7 +503,7 @@ static mvs_status autotune_lanes(mvs_ctx* c, int32_t ref, const int32_t* srcs, i
     int best = cand[0];
     for (int lanes : cand) {
         rc.lanes_hint = lanes;
-        CK(c, use_workspace(c, rc, n, &q, 4));   // the stored windows follow the layout
+        CK(c, use_workspace(c, &rc, 1, n, &q, 4));   // the stored windows follow the layout
         if (rc.win) CK(c, launch_windows(rc, c->stream));
         for (int rep = 0; rep < 2; ++rep) {   // the first run warms caches and launch configuration
             CK(c, cudaMemcpyAsync(V.plane, keep, n * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream));
@@ -564,7 +582,7 @@ mvs_status mvs_patchmatch_batch(mvs_ctx* c, int32_t n_ref, const int32_t* refs, 
     }
     size_t most = 0;
     for (auto& rc : rcs) most = std::max(most, (size_t)rc.W * rc.H);
-    for (auto& rc : rcs) CK(c, use_workspace(c, rc, most, p, pend - p->phase_begin));
+    CK(c, use_workspace(c, rcs.data(), n_ref, most, p, pend - p->phase_begin));
     std::vector<int32_t> kr(refs, refs + n_ref), ks(srcs, srcs + (size_t)n_ref * n_src);
     // a graph captured for the same call, else the least recently used slot
     BatchGraph* hit = nullptr;

@@ -1,0 +1,52 @@
+// Device memory that a context keeps for the checkerboard phases, and how it
+// grows (no counterpart in the paper).  Host code only, with the allocator as
+// a parameter, so that the rules can be checked without a GPU:
+//   void* get(size_t)   device memory, or null
+//   bool full()         the last get failed because the memory is used up
+//   void put(void*)     gives it back once the work enqueued on it is done
+#pragma once
+#include <cstddef>
+#include <cstdint>
+
+struct WsBuffer {
+    void* p = nullptr;
+    size_t bytes = 0;
+};
+
+struct PhaseWorkspace {
+    WsBuffer draws;      // the refinement perturbations of an iteration
+    WsBuffer windows;    // the stored windows
+    size_t limit = (size_t)16 << 30;   // most bytes of stored windows
+    size_t refused = SIZE_MAX;         // windows of this many bytes or more did not fit
+};
+
+// Makes `draws` bytes and, when they can be had, `windows` bytes ready for one
+// call; false when the first cannot.  *stored: whether the windows are there.
+// The caller takes the two pointers once, for all views of the call.  A buffer
+// that is large enough stays where it is, so that a call of the same size
+// costs nothing and the graph captured for it stays valid; a larger one is
+// there before the smaller one goes; windows that did not fit are not asked
+// for again.
+template <class A>
+bool ws_reserve(PhaseWorkspace& w, size_t draws, size_t windows, bool* stored, A& a) {
+    *stored = false;
+    if (w.draws.bytes < draws) {
+        void* p = a.get(draws);
+        if (!p) return false;
+        if (w.draws.p) a.put(w.draws.p);
+        w.draws = WsBuffer{p, draws};
+    }
+    if (windows == 0 || windows > w.limit) return true;
+    if (w.windows.bytes < windows) {
+        if (windows >= w.refused) return true;
+        void* p = a.get(windows);
+        if (!p) {
+            if (a.full()) w.refused = windows;
+            return true;
+        }
+        if (w.windows.p) a.put(w.windows.p);
+        w.windows = WsBuffer{p, windows};
+    }
+    *stored = true;
+    return true;
+}
