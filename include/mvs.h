@@ -176,13 +176,23 @@ const char* mvs_last_error(const mvs_ctx* ctx);
  *   The context keeps a workspace for its largest view: 20 bytes per pixel
  *   and, when the call initialises or runs at least two iterations, each
  *   pixel's reference window (8 bytes per sample slot and 64 more, 1088 bytes
- *   for 11 x 11 samples) if all of them take at most 16 GiB and fit the device;
- *   otherwise the windows are rebuilt at every visit, with the same results.
+ *   for 11 x 11 samples) if all of them take at most half of the device memory
+ *   that is free then and no more than mvs_window_limit allows; otherwise the
+ *   windows are rebuilt at every visit, with the same results.  The windows
+ *   give way when the context needs memory for anything else.
  * Errors: MVS_EINVAL (bad index, duplicate or self source, n_src outside
  *   1..32, window outside 2..22 samples, d_lo >= d_hi, NULL buffers),
  *   MVS_EUNSUPPORTED (precision other than 0 or 1), MVS_ENOMEM, MVS_ECUDA. */
 mvs_status mvs_patchmatch(mvs_ctx* ctx, int32_t ref, const int32_t* srcs, int32_t n_src,
                           const mvs_pm_params* params, mvs_depth_map* out);
+
+/* Most bytes of device memory that the context's stored windows may take
+ * (see mvs_patchmatch; 16 GiB unless set).  0: none, every visit rebuilds its
+ * window.  Windows kept beyond the new limit are given back before the call
+ * returns (it then waits for the context's stream).  Results do not depend on
+ * it.
+ * Errors: MVS_EINVAL (NULL ctx, negative limit), MVS_ECUDA. */
+mvs_status mvs_window_limit(mvs_ctx* ctx, int64_t bytes);
 
 /* Depth maps of several reference views in one call: for each view in
  * turn, its initialisation and its half-iterations in the phase range

@@ -119,6 +119,38 @@ void rel_pose(const mvs_camera& r, const mvs_camera& j, double* Rr, double* tr) 
     for (int a = 0; a < 3; ++a) tr[a] = j.t[a] - (Rr[3 * a] * r.t[0] + Rr[3 * a + 1] * r.t[1] + Rr[3 * a + 2] * r.t[2]);
 }
 
+// device memory of a context (the allocator of workspace.h)
+struct CtxMemory {
+    mvs_ctx* c;
+    cudaError_t err = cudaSuccess;   // of the last get
+    void* get(size_t bytes) {
+        void* p = nullptr;
+        err = cudaMalloc(&p, bytes);
+        if (err == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
+    }
+    bool full() const { return err == cudaErrorMemoryAllocation; }
+    void put(void* p) {
+        cudaStreamSynchronize(c->stream);
+        cudaFree(p);
+    }
+    size_t available() const {
+        size_t free = 0, total = 0;
+        if (cudaMemGetInfo(&free, &total) == cudaSuccess) return free;
+        cudaGetLastError();
+        return 0;
+    }
+};
+
+// memory of a context other than its stored windows, which give way to it
+template <class T>
+cudaError_t ctx_malloc(mvs_ctx* c, T** p, size_t bytes) {
+    CtxMemory mem{c};
+    *p = (T*)ws_get(c->work, bytes, mem);
+    return mem.err;
+}
+
 void* scratch(mvs_ctx* c, int slot, size_t bytes, cudaError_t* e) {
     Scratch& s = c->scratch[slot];
     *e = cudaSuccess;
@@ -129,8 +161,8 @@ void* scratch(mvs_ctx* c, int slot, size_t bytes, cudaError_t* e) {
         s.p = nullptr;
         s.bytes = 0;
     }
-    *e = cudaMalloc(&s.p, bytes);
-    if (*e != cudaSuccess) { s.p = nullptr; return nullptr; }
+    *e = ctx_malloc(c, &s.p, bytes);
+    if (*e != cudaSuccess) return nullptr;
     s.bytes = bytes;
     return s.p;
 }
@@ -260,37 +292,19 @@ mvs_status ensure_map(mvs_ctx* c, int32_t v) {
     ViewData& V = c->views[v];
     if (V.plane) return MVS_OK;
     size_t n = (size_t)V.cam.width * V.cam.height;
-    CK(c, cudaMalloc(&V.plane, n * sizeof(float4)));
-    CK(c, cudaMalloc(&V.cost, n * sizeof(float)));
-    CK(c, cudaMalloc(&V.memo, n * MVS_MEMO_WORDS * sizeof(uint32_t)));
-    CK(c, cudaMalloc(&V.gen, n * sizeof(uint32_t)));
+    CK(c, ctx_malloc(c, &V.plane, n * sizeof(float4)));
+    CK(c, ctx_malloc(c, &V.cost, n * sizeof(float)));
+    CK(c, ctx_malloc(c, &V.memo, n * MVS_MEMO_WORDS * sizeof(uint32_t)));
+    CK(c, ctx_malloc(c, &V.gen, n * sizeof(uint32_t)));
     CK(c, cudaMemsetAsync(V.gen, 0, n * sizeof(uint32_t), c->stream));
     return MVS_OK;
 }
-
-// device memory of a context's workspace
-struct CtxMemory {
-    mvs_ctx* c;
-    cudaError_t err = cudaSuccess;   // of the last get
-    void* get(size_t bytes) {
-        void* p = nullptr;
-        err = cudaMalloc(&p, bytes);
-        if (err == cudaSuccess) return p;
-        cudaGetLastError();
-        return nullptr;
-    }
-    bool full() const { return err == cudaErrorMemoryAllocation; }
-    void put(void* p) {
-        cudaStreamSynchronize(c->stream);
-        cudaFree(p);
-    }
-};
 
 // The phases' workspace, one per context (its views run one after another):
 // the refinement perturbations of an iteration (20 bytes per pixel) and, when
 // the call visits every pixel often enough to pay for storing the windows (an
 // initialisation, which builds them anyway, or at least two iterations) and
-// they fit, the stored windows; otherwise the phases rebuild each window, with
+// workspace.h lets them have the memory, the stored windows; otherwise the phases rebuild each window, with
 // the same results.  One choice for all n views of a call, of at most
 // max_pixels pixels each and with the same window.
 cudaError_t use_workspace(mvs_ctx* c, RefConst* rcs, int n, size_t max_pixels, const mvs_pm_params* p, int phases) {
@@ -465,6 +479,17 @@ mvs_status mvs_patchmatch(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t 
     CK(c, cudaMemcpyAsync(out->plane, V.plane, n * sizeof(float4), kind_out(out->mem), c->stream));
     CK(c, cudaMemcpyAsync(out->cost, V.cost, n * sizeof(float), kind_out(out->mem), c->stream));
     if (out->mem == MVS_MEM_HOST) CK(c, cudaStreamSynchronize(c->stream));
+    return MVS_OK;
+}
+
+mvs_status mvs_window_limit(mvs_ctx* c, int64_t bytes) {
+    if (!c) return MVS_EINVAL;
+    if (bytes < 0) return fail(c, MVS_EINVAL, "limit must not be negative");
+    CK(c, cudaSetDevice(c->device));
+    c->work.limit = (size_t)bytes;
+    c->work.refused = SIZE_MAX;
+    CtxMemory mem{c};
+    if (c->work.windows.bytes > c->work.limit) ws_drop_windows(c->work, mem);
     return MVS_OK;
 }
 

@@ -4,6 +4,7 @@
 //   void* get(size_t)   device memory, or null
 //   bool full()         the last get failed because the memory is used up
 //   void put(void*)     gives it back once the work enqueued on it is done
+//   size_t available()  free bytes of the device
 #pragma once
 #include <cstddef>
 #include <cstdint>
@@ -17,34 +18,53 @@ struct PhaseWorkspace {
     WsBuffer draws;      // the refinement perturbations of an iteration
     WsBuffer windows;    // the stored windows
     size_t limit = (size_t)16 << 30;   // most bytes of stored windows
-    size_t refused = SIZE_MAX;         // windows of this many bytes or more did not fit
+    size_t refused = SIZE_MAX;         // windows of this many bytes or more did not fit, although they seemed to
 };
+
+// The windows go back: only later calls of this context would read them.
+template <class A>
+void ws_drop_windows(PhaseWorkspace& w, A& a) {
+    if (w.windows.p) a.put(w.windows.p);
+    w.windows = WsBuffer();
+}
+
+// Device memory for anything else of the context: the windows give way to it.
+template <class A>
+void* ws_get(PhaseWorkspace& w, size_t bytes, A& a) {
+    void* p = a.get(bytes);
+    if (!p && a.full() && w.windows.p) {
+        ws_drop_windows(w, a);
+        p = a.get(bytes);
+    }
+    return p;
+}
 
 // Makes `draws` bytes and, when they can be had, `windows` bytes ready for one
 // call; false when the first cannot.  *stored: whether the windows are there.
 // The caller takes the two pointers once, for all views of the call.  A buffer
 // that is large enough stays where it is, so that a call of the same size
 // costs nothing and the graph captured for it stays valid; a larger one is
-// there before the smaller one goes; windows that did not fit are not asked
-// for again.
+// there before the smaller one goes.  The windows take at most half of what is
+// free, so that the rest of the process finds memory too; asking first also
+// spares the calls on a full device an allocation that fails.
 template <class A>
 bool ws_reserve(PhaseWorkspace& w, size_t draws, size_t windows, bool* stored, A& a) {
     *stored = false;
     if (w.draws.bytes < draws) {
-        void* p = a.get(draws);
+        void* p = ws_get(w, draws, a);
         if (!p) return false;
         if (w.draws.p) a.put(w.draws.p);
         w.draws = WsBuffer{p, draws};
     }
     if (windows == 0 || windows > w.limit) return true;
     if (w.windows.bytes < windows) {
-        if (windows >= w.refused) return true;
+        if (windows >= w.refused || windows > (a.available() + w.windows.bytes) / 2) return true;
         void* p = a.get(windows);
         if (!p) {
             if (a.full()) w.refused = windows;
             return true;
         }
-        if (w.windows.p) a.put(w.windows.p);
+        ws_drop_windows(w, a);
         w.windows = WsBuffer{p, windows};
     }
     *stored = true;

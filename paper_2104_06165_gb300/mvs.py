@@ -147,6 +147,8 @@ def load():
     L.mvs_last_error.argtypes = [vp]
     L.mvs_patchmatch.restype = i32
     L.mvs_patchmatch.argtypes = [vp, i32, ip, i32, C.POINTER(mvs_pm_params), C.POINTER(mvs_depth_map)]
+    L.mvs_window_limit.restype = i32
+    L.mvs_window_limit.argtypes = [vp, C.c_int64]
     L.mvs_patchmatch_batch.restype = i32
     L.mvs_patchmatch_batch.argtypes = [vp, i32, ip, ip, i32, C.POINTER(mvs_pm_params), C.POINTER(mvs_depth_map)]
     L.mvs_plane_cost.restype = i32
@@ -291,6 +293,11 @@ def mvs_patchmatch(ctx, ref, srcs, params: PMParams, plane, cost):
     out = mvs_depth_map(pp, cp, mem)
     cpar = params.c()
     _check(load().mvs_patchmatch(ctx, ref, s, ns, C.byref(cpar), C.byref(out)), ctx)
+
+
+def mvs_window_limit(ctx, limit):
+    """Most bytes of device memory for the context's stored windows (0: none)."""
+    _check(load().mvs_window_limit(ctx, int(limit)), ctx)
 
 
 def mvs_patchmatch_batch(ctx, refs, srcs, params: PMParams, planes, costs):

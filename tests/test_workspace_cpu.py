@@ -35,16 +35,27 @@ struct Fake {
         return p;
     }
     bool full() const { return failed; }
+    size_t hidden = 0;                  // free bytes that cannot be had in one piece
+    size_t available() const { return room - used() + hidden; }
     void put(void* p) { puts++; if (!live.erase(p)) { std::puts("put of a dead pointer"); std::exit(2); } }
 };
-// arguments: room, limit, then "draws windows" per call
+// arguments: room, limit, then "draws windows" per call; draws < 0: that much
+// for something else of the context (windows: free bytes that cannot be had)
 int main(int argc, char** argv) {
     Fake a{(size_t)std::atoll(argv[1])};
     PhaseWorkspace w;
     w.limit = (size_t)std::atoll(argv[2]);
     for (int i = 3; i + 1 < argc; i += 2) {
-        const size_t draws = std::atoll(argv[i]), windows = std::atoll(argv[i + 1]);
+        const long long d = std::atoll(argv[i]);
+        const size_t draws = d < 0 ? 0 : d, windows = std::atoll(argv[i + 1]);
         bool stored = false;
+        if (d < 0) {
+            a.hidden = windows;
+            const bool got = d == -1 || ws_get(w, -d, a) != nullptr;
+            std::printf("%d 0 1 %d %d %d %zu %zu %zu\n", (int)got, a.gets, a.fails, a.puts, (size_t)w.draws.p,
+                        (size_t)w.windows.p, a.used());
+            continue;
+        }
         const bool ok = ws_reserve(w, draws, windows, &stored, a);
         const bool fits = ok && a.live.count(w.draws.p) && a.live[w.draws.p] >= draws &&
                           (!stored || (a.live.count(w.windows.p) && a.live[w.windows.p] >= windows));
@@ -76,23 +87,41 @@ def test_a_call_that_fits_changes_nothing(workspace):
     assert all(c[3:] == r[0][3:] for c in r) and r[0][3:6] == (2, 0, 0)
 
 
-def test_windows_without_room_cost_one_failed_allocation(workspace):
+def test_windows_without_room_cost_nothing(workspace):
     """Views of one call share one choice, and calls after the first allocate
     and free nothing: the perturbations stay where the captured graph has them."""
     r = workspace(900, 1 << 40, (20, 1000), (20, 1000), (10, 2000), (20, 1000))
     assert [c[:3] for c in r] == [(1, 0, 1)] * 4
-    assert all(c[3:] == r[0][3:] for c in r) and r[0][4:6] == (1, 0)
+    assert all(c[3:] == r[0][3:] for c in r) and r[0][4:6] == (0, 0)
     # smaller windows that fit are stored all the same
-    r = workspace(900, 1 << 40, (20, 1000), (20, 500), (20, 1000), (20, 500))
+    r = workspace(900, 1 << 40, (20, 1000), (20, 400), (20, 1000), (20, 400))
     assert [c[1] for c in r] == [0, 1, 0, 1] and r[3][6:] == r[1][6:]
+    # free memory that turns out not to be there is asked for once
+    r = workspace(900, 1 << 40, (-1, 5000), (20, 1000), (20, 1000), (20, 2000), (20, 800))
+    assert [c[1] for c in r] == [0, 0, 0, 0, 1] and [c[4] for c in r] == [0, 1, 1, 1, 1]
 
 
 def test_the_larger_buffer_is_there_before_the_smaller_one_goes(workspace):
     r = workspace(10000, 1 << 40, (20, 1000), (40, 3000))
     assert r[1][:3] == (1, 1, 1) and r[1][5] == 2 and r[1][8] == 3040
     # no room for a larger one: the smaller windows stay for the smaller views
-    r = workspace(1500, 1 << 40, (20, 1000), (20, 1400), (20, 1000))
+    r = workspace(1500, 1 << 40, (20, 700), (20, 1400), (20, 700))
     assert [c[1] for c in r] == [1, 0, 1] and r[2][7] == r[0][7] and r[2][5] == 0
+
+
+def test_windows_take_half_of_what_is_free_and_give_way(workspace):
+    r = workspace(2020, 1 << 40, (20, 1001), (20, 1000))
+    assert [c[1] for c in r] == [0, 1]
+    # something else of the context needs more than is left
+    r = workspace(2020, 1 << 40, (20, 1000), (-1500, 0), (20, 1000), (20, 250))
+    assert [c[0] for c in r] == [1, 1, 1, 1] and [c[1] for c in r] == [1, 0, 0, 1]
+    assert r[1][7] == 0 and r[1][8] == 1520
+    # also the perturbations of a larger view
+    r = workspace(2020, 1 << 40, (20, 1000), (1200, 0))
+    assert r[1][0] == 1 and r[1][7] == 0
+    # more than there is: refused, and what was there stays usable
+    r = workspace(2020, 1 << 40, (20, 0), (-5000, 0), (20, 0))
+    assert [c[0] for c in r] == [1, 0, 1] and r[2][6] == r[0][6]
 
 
 def test_limit_and_no_room_at_all(workspace):
