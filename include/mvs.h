@@ -179,7 +179,10 @@ const char* mvs_last_error(const mvs_ctx* ctx);
  *   for 11 x 11 samples) if all of them take at most half of the device memory
  *   that is free then and no more than mvs_window_limit allows; otherwise the
  *   windows are rebuilt at every visit, with the same results.  The windows
- *   give way when the context needs memory for anything else.
+ *   give way when the context needs memory for anything else.  A call can be
+ *   captured into a graph of the caller (device buffers) once a call for a
+ *   view of at least that size has run; the workspace that a captured call
+ *   uses then stays until mvs_destroy, also when later calls need a larger one.
  * Errors: MVS_EINVAL (bad index, duplicate or self source, n_src outside
  *   1..32, window outside 2..22 samples, d_lo >= d_hi, NULL buffers),
  *   MVS_EUNSUPPORTED (precision other than 0 or 1), MVS_ENOMEM, MVS_ECUDA. */

@@ -141,6 +141,11 @@ struct CtxMemory {
         cudaGetLastError();
         return 0;
     }
+    bool capturing() const {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+        return st != cudaStreamCaptureStatusNone;
+    }
 };
 
 // memory of a context other than its stored windows, which give way to it
@@ -407,6 +412,7 @@ void mvs_destroy(mvs_ctx* c) {
     for (auto& s : c->scratch) cudaFree(s.p);
     cudaFree(c->work.draws.p);
     cudaFree(c->work.windows.p);
+    for (void* p : c->work.retired) cudaFree(p);
     for (auto e : c->ev) cudaEventDestroy(e);
     cudaFree(c->evals);
     cudaFreeHost(c->wait_status);
@@ -489,7 +495,7 @@ mvs_status mvs_window_limit(mvs_ctx* c, int64_t bytes) {
     c->work.limit = (size_t)bytes;
     c->work.refused = SIZE_MAX;
     CtxMemory mem{c};
-    if (c->work.windows.bytes > c->work.limit) ws_drop_windows(c->work, mem);
+    if (c->work.windows.bytes > c->work.limit) ws_release(c->work, c->work.windows, mem);
     return MVS_OK;
 }
 

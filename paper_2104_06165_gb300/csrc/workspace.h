@@ -5,13 +5,16 @@
 //   bool full()         the last get failed because the memory is used up
 //   void put(void*)     gives it back once the work enqueued on it is done
 //   size_t available()  free bytes of the device
+//   bool capturing()    the call is being captured into a graph of the caller
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 
 struct WsBuffer {
     void* p = nullptr;
     size_t bytes = 0;
+    bool captured = false;   // a graph of the caller may read it
 };
 
 struct PhaseWorkspace {
@@ -19,21 +22,24 @@ struct PhaseWorkspace {
     WsBuffer windows;    // the stored windows
     size_t limit = (size_t)16 << 30;   // most bytes of stored windows
     size_t refused = SIZE_MAX;         // windows of this many bytes or more did not fit, although they seemed to
+    std::vector<void*> retired;        // replaced buffers of captured calls, kept as long as the context
 };
 
-// The windows go back: only later calls of this context would read them.
+// Takes a buffer out of use: only later calls of this context would use it,
+// or a graph that the caller captured a call into.
 template <class A>
-void ws_drop_windows(PhaseWorkspace& w, A& a) {
-    if (w.windows.p) a.put(w.windows.p);
-    w.windows = WsBuffer();
+void ws_release(PhaseWorkspace& w, WsBuffer& b, A& a) {
+    if (b.captured) w.retired.push_back(b.p);
+    else if (b.p) a.put(b.p);
+    b = WsBuffer();
 }
 
 // Device memory for anything else of the context: the windows give way to it.
 template <class A>
 void* ws_get(PhaseWorkspace& w, size_t bytes, A& a) {
     void* p = a.get(bytes);
-    if (!p && a.full() && w.windows.p) {
-        ws_drop_windows(w, a);
+    if (!p && a.full() && w.windows.p && !w.windows.captured) {
+        ws_release(w, w.windows, a);
         p = a.get(bytes);
     }
     return p;
@@ -53,20 +59,25 @@ bool ws_reserve(PhaseWorkspace& w, size_t draws, size_t windows, bool* stored, A
     if (w.draws.bytes < draws) {
         void* p = ws_get(w, draws, a);
         if (!p) return false;
-        if (w.draws.p) a.put(w.draws.p);
-        w.draws = WsBuffer{p, draws};
+        ws_release(w, w.draws, a);
+        w.draws.p = p;
+        w.draws.bytes = draws;
     }
+    const bool capturing = a.capturing();   // (nothing can be allocated then)
+    w.draws.captured |= capturing;
     if (windows == 0 || windows > w.limit) return true;
     if (w.windows.bytes < windows) {
-        if (windows >= w.refused || windows > (a.available() + w.windows.bytes) / 2) return true;
+        if (capturing || windows >= w.refused || windows > (a.available() + w.windows.bytes) / 2) return true;
         void* p = a.get(windows);
         if (!p) {
             if (a.full()) w.refused = windows;
             return true;
         }
-        ws_drop_windows(w, a);
-        w.windows = WsBuffer{p, windows};
+        ws_release(w, w.windows, a);
+        w.windows.p = p;
+        w.windows.bytes = windows;
     }
+    w.windows.captured |= capturing;
     *stored = true;
     return true;
 }

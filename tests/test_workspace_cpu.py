@@ -36,11 +36,14 @@ struct Fake {
     }
     bool full() const { return failed; }
     size_t hidden = 0;                  // free bytes that cannot be had in one piece
+    bool captures = false;
+    bool capturing() const { return captures; }
     size_t available() const { return room - used() + hidden; }
     void put(void* p) { puts++; if (!live.erase(p)) { std::puts("put of a dead pointer"); std::exit(2); } }
 };
 // arguments: room, limit, then "draws windows" per call; draws < 0: that much
-// for something else of the context (windows: free bytes that cannot be had)
+// for something else of the context (-1: free bytes that cannot be had, -2:
+// whether the calls are captured)
 int main(int argc, char** argv) {
     Fake a{(size_t)std::atoll(argv[1])};
     PhaseWorkspace w;
@@ -50,8 +53,9 @@ int main(int argc, char** argv) {
         const size_t draws = d < 0 ? 0 : d, windows = std::atoll(argv[i + 1]);
         bool stored = false;
         if (d < 0) {
-            a.hidden = windows;
-            const bool got = d == -1 || ws_get(w, -d, a) != nullptr;
+            if (d == -1) a.hidden = windows;
+            if (d == -2) a.captures = windows != 0;
+            const bool got = d >= -2 || ws_get(w, -d, a) != nullptr;
             std::printf("%d 0 1 %d %d %d %zu %zu %zu\n", (int)got, a.gets, a.fails, a.puts, (size_t)w.draws.p,
                         (size_t)w.windows.p, a.used());
             continue;
@@ -122,6 +126,20 @@ def test_windows_take_half_of_what_is_free_and_give_way(workspace):
     # more than there is: refused, and what was there stays usable
     r = workspace(2020, 1 << 40, (20, 0), (-5000, 0), (20, 0))
     assert [c[0] for c in r] == [1, 0, 1] and r[2][6] == r[0][6]
+
+
+def test_what_a_captured_call_uses_stays(workspace):
+    # captured, then a larger call: new buffers, and nothing goes back
+    r = workspace(9000, 1 << 40, (20, 1000), (-2, 1), (20, 1000), (-2, 0), (40, 2000), (40, 3000))
+    assert r[2][:3] == (1, 1, 1) and r[2][6:8] == r[0][6:8]
+    assert r[4][5] == 0 and r[4][8] == 20 + 1000 + 40 + 2000
+    assert r[5][5] == 1 and r[5][8] == 20 + 1000 + 40 + 3000     # the later ones were not captured
+    # nothing is allocated during a capture: without room for the windows they are rebuilt
+    r = workspace(9000, 1 << 40, (20, 0), (-2, 1), (20, 1000), (20, 1000))
+    assert [c[1] for c in r] == [0, 0, 0, 0] and r[3][3] == r[0][3]
+    # windows of a captured call give way to nothing
+    r = workspace(2020, 1 << 40, (20, 0), (20, 900), (-2, 1), (20, 900), (-2, 0), (-1500, 0))
+    assert [c[0] for c in r] == [1, 1, 1, 1, 1, 0] and r[5][7] == r[1][7]
 
 
 def test_limit_and_no_room_at_all(workspace):
