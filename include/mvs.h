@@ -341,9 +341,14 @@ mvs_status mvs_sparse_depth_range(mvs_ctx* ctx, int32_t ref, int64_t n_points, c
  *   context's copy of the view is updated.  pm gives the window / ZNCC
  *   parameters for the hypothesis costs.
  * Errors: MVS_ESTATE if the view has no depth map, MVS_EINVAL (also for an
- *   unknown selection), MVS_ECUDA, MVS_ETIMEOUT once a bounded wait of the
- *   message passing ran out (with host buffers by this call, else by the next
- *   one; mvs_phi_mrf likewise). */
+ *   unknown selection), MVS_ECUDA, MVS_ETIMEOUT when a bounded wait of the
+ *   message passing ran out (about a second).  Nothing is filled then: the
+ *   view's map is the one given, mvs_phi_mrf's labels are all -2.  With host
+ *   buffers the call itself reports it.  With device buffers the first
+ *   mvs_plane_infer, mvs_phi_mrf, mvs_geo_filter, mvs_fuse or mvs_propose of
+ *   the context that is made after it happened does, once, instead of its own
+ *   work; mvs_fuse and calls with host buffers also report what has happened
+ *   by the time they have synchronised. */
 mvs_status mvs_plane_infer(mvs_ctx* ctx, int32_t ref, const int32_t* srcs, int32_t n_src,
                            const mvs_pm_params* pm, const mvs_phi_params* phi, const uint8_t* keep_mask,
                            mvs_depth_map* inout);
@@ -379,6 +384,14 @@ mvs_status mvs_phi_select(mvs_ctx* ctx, int32_t ref, const uint8_t* known, const
                           const uint8_t* valid, const int32_t* label, float* plane, int32_t mem);
 mvs_status mvs_phi_select_min_cost(mvs_ctx* ctx, int32_t ref, const uint8_t* known, const float* hyp,
                                    const uint8_t* valid, const float* hcost, float* plane, int32_t mem);
+
+/* Makes the next message passing of the context (mvs_phi_mrf, or
+ * mvs_plane_infer with the MRF) leave out its first eight node rows, so that
+ * the wait for them runs out, after about a millisecond: a check of that path,
+ * no counterpart in the paper.  (Needs several-label nodes on both sides of
+ * node rows 7 and 8; else nothing waits and the labels are unspecified.)
+ * Errors: MVS_EINVAL for a NULL ctx. */
+mvs_status mvs_phi_test_timeout(mvs_ctx* ctx);
 
 /* Allocation-free variant of mvs_phi_hypotheses (the paper has no
  * counterpart; this is a deployment convenience).

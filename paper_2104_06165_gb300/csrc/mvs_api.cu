@@ -65,6 +65,7 @@ struct mvs_ctx {
     size_t ev_used = 0;
     long long launches0 = 0;
     int* wait_status = nullptr;            // host memory the kernels write: MVS_DEV_TIMEOUT once a wait ran out
+    bool test_timeout = false;             // the next message passing gives up (mvs_phi_test_timeout)
     unsigned long long* evals = nullptr;   // device counter of evaluated (pixel, hypothesis, view)
     // batched path
     cudaStream_t gstream = nullptr;        // private stream for graph capture / replay
@@ -172,17 +173,20 @@ void* scratch(mvs_ctx* c, int slot, size_t bytes, cudaError_t* e) {
     return s.p;
 }
 
-// MVS_ETIMEOUT once a bounded wait of this context's kernels ran out since the
-// last check: at the next call that uses them, or at once for host outputs
+// MVS_ETIMEOUT once a bounded wait of this context's message passing ran out
+// since the last check.  Every call that reads a stored map or passes messages
+// checks before it does anything, and again after it has synchronised.
 mvs_status check_waits(mvs_ctx* c) {
-    if (!c->wait_status) {
-        CK(c, cudaHostAlloc((void**)&c->wait_status, sizeof(int), cudaHostAllocDefault));
-        *c->wait_status = 0;
-    }
     volatile int* st = c->wait_status;
-    if (*st == 0) return MVS_OK;
+    if (!st || *st == 0) return MVS_OK;
     *st = 0;
-    return fail(c, MVS_ETIMEOUT, "message passing gave up waiting for the row above");
+    return fail(c, MVS_ETIMEOUT, "message passing gave up waiting for the row above; its map was not filled");
+}
+mvs_status ensure_wait_status(mvs_ctx* c) {
+    if (c->wait_status) return MVS_OK;
+    CK(c, cudaHostAlloc((void**)&c->wait_status, sizeof(int), cudaHostAllocDefault));
+    *c->wait_status = 0;
+    return MVS_OK;
 }
 
 // true when p is device (or managed) memory the kernels can read
@@ -751,6 +755,7 @@ mvs_status mvs_geo_filter(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t 
     if (!c->views[ref].has_map) return fail(c, MVS_ESTATE, "view %d has no depth map", ref);
     for (int i = 0; i < n_src; ++i)
         if (!c->views[srcs[i]].has_map) return fail(c, MVS_ESTATE, "source view %d has no depth map", srcs[i]);
+    if ((st = check_waits(c)) != MVS_OK) return st;
     CK(c, cudaSetDevice(c->device));
     const ViewData& V = c->views[ref];
     FilterConst fc;
@@ -791,6 +796,7 @@ mvs_status mvs_geo_filter(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t 
         CK(c, cudaMemcpyAsync(keep_mask, keep_d, n, cudaMemcpyDeviceToHost, c->stream));
         if (count) CK(c, cudaMemcpyAsync(count, cnt_d, n * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
+        return check_waits(c);
     }
     return MVS_OK;
 }
@@ -813,6 +819,8 @@ mvs_status mvs_fuse(mvs_ctx* c, int32_t n_views, const int32_t* views, const uin
         if (K[3] != 0.0 || K[6] != 0.0 || K[7] != 0.0 || K[8] != 1.0)
             return fail(c, MVS_EUNSUPPORTED, "view %d: fusion needs a pinhole K = [fx s cx; 0 fy cy; 0 0 1]", v);
     }
+    mvs_status ws = check_waits(c);
+    if (ws != MVS_OK) return ws;
     CK(c, cudaSetDevice(c->device));
     // scratch slot 6, every region starting on a 16-byte boundary: per view
     // the claim and depth arrays (and a device copy of a host keep mask),
@@ -896,6 +904,7 @@ mvs_status mvs_fuse(mvs_ctx* c, int32_t n_views, const int32_t* views, const uin
     long long tot = 0;
     CK(c, cudaMemcpyAsync(&tot, total, sizeof tot, cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
+    if ((ws = check_waits(c)) != MVS_OK) return ws;
     *n_points = tot;
     const long long nw = std::min<long long>(tot, capacity);
     if (mem == MVS_MEM_HOST && (nw > 0 || owner)) {
@@ -1138,7 +1147,8 @@ mvs_status mvs_phi_mrf(mvs_ctx* c, int32_t W, int32_t H, const uint8_t* known, c
         return fail(c, MVS_EINVAL, "need kappa1 > 0, kappa2 > 0, kappa3 > 1");
     if (mem != MVS_MEM_DEVICE && mem != MVS_MEM_HOST) return fail(c, MVS_EINVAL, "bad mem kind");
     CK(c, cudaSetDevice(c->device));
-    mvs_status ws = check_waits(c);
+    mvs_status ws = ensure_wait_status(c);
+    if (ws == MVS_OK) ws = check_waits(c);
     if (ws != MVS_OK) return ws;
     size_t n = (size_t)W * H;
     int gw = (W + 1) / 2, gh = (H + 1) / 2;
@@ -1168,8 +1178,11 @@ mvs_status mvs_phi_mrf(mvs_ctx* c, int32_t W, int32_t H, const uint8_t* known, c
         CK(c, cudaMemcpyAsync(v2, valid, n * 4, cudaMemcpyHostToDevice, c->stream));
         kd = k2; dd = d2; hd = h2; vd = v2; cd = c2; ld = l2;
     }
+    const bool test_timeout = c->test_timeout;
+    const int* gave_up = nullptr;
+    c->test_timeout = false;
     CK(c, launch_phi_mrf(W, H, kd, dd, hd, vd, cd, phi->kappa1, phi->kappa2, phi->kappa3, phi->trw_iters, ld, work,
-                         c->wait_status, c->stream));
+                         c->wait_status, test_timeout, &gave_up, c->stream));
     if (mem == MVS_MEM_HOST) {
         CK(c, cudaMemcpyAsync(label, ld, g * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
@@ -1219,7 +1232,7 @@ mvs_status mvs_phi_select(mvs_ctx* c, int32_t ref, const uint8_t* known, const f
         CK(c, cudaMemcpyAsync(v2, valid, n * 4, cudaMemcpyHostToDevice, c->stream));
         kd = k2; hd = h2; vd = v2; ld = l2; pd = p2;
     }
-    CK(c, launch_phi_select(rc, kd, hd, vd, ld, pd, newd, c->stream));
+    CK(c, launch_phi_select(rc, kd, hd, vd, ld, pd, newd, nullptr, c->stream));
     if (mem == MVS_MEM_HOST) {
         CK(c, cudaMemcpyAsync(plane, pd, n * sizeof(float4), cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
@@ -1291,7 +1304,7 @@ mvs_status mvs_plane_infer(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t
     if (phi->selection != MVS_PHI_SELECT_MRF && phi->selection != MVS_PHI_SELECT_MIN_COST)
         return fail(c, MVS_EINVAL, "unknown selection %d", (int)phi->selection);
     CK(c, cudaSetDevice(c->device));
-    if ((st = check_waits(c)) != MVS_OK) return st;
+    if ((st = ensure_wait_status(c)) != MVS_OK || (st = check_waits(c)) != MVS_OK) return st;
     if ((st = ensure_map(c, ref)) != MVS_OK) return st;
     ViewData& V = c->views[ref];
     int W = V.cam.width, H = V.cam.height;
@@ -1331,9 +1344,12 @@ mvs_status mvs_plane_infer(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t
     if (phi->selection == MVS_PHI_SELECT_MIN_COST) {
         CK(c, launch_phi_select_min_cost(rc, known, hyp, valid, hcost, V.plane, newd, c->stream));
     } else {
+        const bool test_timeout = c->test_timeout;
+        const int* gave_up = nullptr;
+        c->test_timeout = false;
         CK(c, launch_phi_mrf(W, H, known, depth, hyp, valid, hcost, phi->kappa1, phi->kappa2, phi->kappa3,
-                             phi->trw_iters, label, mwork, c->wait_status, c->stream));
-        CK(c, launch_phi_select(rc, known, hyp, valid, label, V.plane, newd, c->stream));
+                             phi->trw_iters, label, mwork, c->wait_status, test_timeout, &gave_up, c->stream));
+        CK(c, launch_phi_select(rc, known, hyp, valid, label, V.plane, newd, gave_up, c->stream));
     }
     V.has_map = true;
     CK(c, cudaMemcpyAsync(inout->plane, V.plane, n * sizeof(float4), kind_out(mem), c->stream));
@@ -1344,6 +1360,12 @@ mvs_status mvs_plane_infer(mvs_ctx* c, int32_t ref, const int32_t* srcs, int32_t
     return MVS_OK;
 }
 
+mvs_status mvs_phi_test_timeout(mvs_ctx* c) {
+    if (!c) return MVS_EINVAL;
+    c->test_timeout = true;
+    return MVS_OK;
+}
+
 mvs_status mvs_propose(mvs_ctx* c, int32_t ref, mvs_cnn* net, float* proposals) {
     mvs_status st = check_view(c, ref);
     if (st != MVS_OK) return st;
@@ -1351,6 +1373,7 @@ mvs_status mvs_propose(mvs_ctx* c, int32_t ref, mvs_cnn* net, float* proposals) 
     if ((uintptr_t)proposals & 15u) return fail(c, MVS_EINVAL, "proposals must be 16-byte aligned");
     ViewData& V = c->views[ref];
     if (!V.has_map) return fail(c, MVS_ESTATE, "view %d has no depth map", ref);
+    if ((st = check_waits(c)) != MVS_OK) return st;
     if (!cnn_shape_ok(net, V.cam.width, V.cam.height))
         return fail(c, MVS_EINVAL, "view size %dx%d is not a multiple of 16 within the network's capacity",
                     V.cam.width, V.cam.height);

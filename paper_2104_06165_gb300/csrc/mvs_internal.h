@@ -162,13 +162,18 @@ size_t phi_line_words(int W, int H);   // scratch of launch_phi_hypotheses, 32-b
 // costs of the hypotheses of every step-th row and column (1: all pixels)
 cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t* valid, float* hcost, int step,
                             cudaStream_t s);
-// status: a word both sides see; MVS_DEV_TIMEOUT once a wait between rows ran out
+// status: a word both sides see; MVS_DEV_TIMEOUT once a wait between rows ran
+// out.  The labels are then -2, and *gave_up, a word of `work`, is set on the
+// device (launch_phi_select leaves the map as it is).  test_timeout makes the
+// wait for the first strip of rows run out.
 cudaError_t launch_phi_mrf(int W, int H, const uint8_t* known, const float* depth, const float* hyp,
                            const uint8_t* valid, const float* hcost, float k1, float k2, float k3, int iters,
-                           int32_t* label, float* work, int* status, cudaStream_t s);
+                           int32_t* label, float* work, int* status, bool test_timeout, const int** gave_up,
+                           cudaStream_t s);
 size_t phi_mrf_work_floats(int W, int H);
 cudaError_t launch_phi_select(const RefConst& rc, const uint8_t* known, const float* hyp, const uint8_t* valid,
-                              const int32_t* label, float4* plane, float* newdepth, cudaStream_t s);
+                              const int32_t* label, float4* plane, float* newdepth, const int* gave_up,
+                              cudaStream_t s);
 cudaError_t launch_phi_select_min_cost(const RefConst& rc, const uint8_t* known, const float* hyp,
                                        const uint8_t* valid, const float* hcost, float4* plane, float* newdepth,
                                        cudaStream_t s);

@@ -168,6 +168,8 @@ def load():
     L.mvs_phi_cost.argtypes = [vp, i32, ip, i32, C.POINTER(mvs_pm_params), fp, u8p, fp, i32]
     L.mvs_phi_mrf.restype = i32
     L.mvs_phi_mrf.argtypes = [vp, i32, i32, u8p, fp, fp, u8p, fp, C.POINTER(mvs_phi_params), vp, i32]
+    L.mvs_phi_test_timeout.restype = i32
+    L.mvs_phi_test_timeout.argtypes = [vp]
     L.mvs_phi_select.restype = i32
     L.mvs_phi_select.argtypes = [vp, i32, u8p, fp, u8p, vp, fp, i32]
     L.mvs_phi_select_min_cost.restype = i32
@@ -428,6 +430,11 @@ def mvs_phi_mrf(ctx, known, depth, hyp, valid, hcost, phi: PhiParams, label):
     b = phi.c()
     _check(load().mvs_phi_mrf(ctx, W, H, _ptr(known)[0], _ptr(depth)[0], _ptr(hyp)[0], _ptr(valid)[0],
                               _ptr(hcost)[0], C.byref(b), _ptr(label)[0], mem), ctx)
+
+
+def mvs_phi_test_timeout(ctx):
+    """The next message passing of the context gives up waiting."""
+    _check(load().mvs_phi_test_timeout(ctx), ctx)
 
 
 def mvs_phi_select(ctx, ref, known, hyp, valid, label, plane):
