@@ -45,9 +45,13 @@ struct Mat3 {
 // with ldmatrix.  A block covers kWgSeg pixels x `rows` image rows and up to 16
 // warps of channel tiles; input rows pass through a ring of four (each is read
 // once per block and used by three output rows), the next row arriving by
-// cp.async while the current one is multiplied.  Bound by shared-memory
-// bandwidth (10 fragment loads per 18 products).  512 x 384, all ten layers:
-// 184 us against 1730 us for the fp32 SIMT reduction it replaces.
+// cp.async while the current one is multiplied.  Bound by the latency of the
+// chain fragment load, product, product with 4 to 16 warps per multiprocessor
+// (128 registers; full-resolution layers: 30 % of the issue slots, 24 to 43 % of
+// the shared-memory pipe) and, on the small levels, by the atomic sums of few
+// blocks.  512 x 384, all ten layers: 184 us against 1730 us for the fp32 SIMT
+// reduction it replaces; the tensor core's fp32 sums differ from its one rounded
+// multiply-add per product by about 2e-6 relative.
 constexpr int kWgSeg = 64;
 struct WgradArgs {
     const bf16* x;
@@ -431,7 +435,8 @@ const int kLayerCout[NL] = {32, 48, 64, 96, 128, 96, 64, 48, 32, 16};
 
 cudaError_t g_cnn_err = cudaSuccess;
 
-// widest level-0 image that is trained on
+// widest level-0 image that training takes (the widest that the layer tests
+// check; no kernel needs the limit)
 constexpr int kMaxTrainWidth = 768;
 
 }  // namespace
@@ -845,14 +850,14 @@ mvs_status mvs_cnn_forward(mvs_cnn* n, const uint8_t* img, const float* plane, c
 mvs_status mvs_cnn_backward(mvs_cnn* n, const uint8_t* img, const float* plane, const float* cost, int32_t W,
                             int32_t H, const float* target, const uint8_t* mask, float* loss_out) {
     if (!n || !img || !plane || !cost || !target || !mask) return MVS_EINVAL;
-    if (W > kMaxTrainWidth) return cnn_fail(n, MVS_EINVAL, "training width above the weight-gradient kernel's limit");
+    if (W > kMaxTrainWidth) return cnn_fail(n, MVS_EINVAL, "training takes images up to 768 pixels wide");
     if ((uintptr_t)target & 15u) return cnn_fail(n, MVS_EINVAL, "target must be 16-byte aligned");
     mvs_status st = run_forward(n, img, (const float4*)plane, cost, W, H);
     if (st != MVS_OK) return st;
     const long long np = (long long)W * H;
     CNK(n, cudaMemsetAsync(n->loss, 0, sizeof(float), n->stream));
-    k_proposal_loss<<<(unsigned)((np + 255) / 256), 256, 0, n->stream>>>(n->y, (const float4*)target, mask, np, n->hc,
-                                                                         1.0f / (float)np, reinterpret_cast<uint4*>(n->gyb), n->loss);
+    k_proposal_loss<<<(unsigned)((np + 255) / 256), 256, 0, n->stream>>>(
+        n->y, (const float4*)target, mask, np, n->hc, 1.0f / (float)np, reinterpret_cast<uint4*>(n->gyb), n->loss);
     count_launch();
     CNK(n, cudaGetLastError());
     CNK(n, cnn_backward(n, W, H));

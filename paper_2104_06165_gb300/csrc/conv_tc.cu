@@ -398,8 +398,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (x.up) {
                     const long long q = ((long long)(2 * py) * (2 * a.W) + 2 * px) * x.up_ch + g0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        reinterpret_cast<uint4*>(x.up)[(q + ((long long)(k >> 1) * (2 * a.W) + (k & 1)) * x.up_ch) / 8 + c] = v;
+                    for (int k = 0; k < 4; ++k) {
+                        const long long at = q + ((long long)(k >> 1) * (2 * a.W) + (k & 1)) * x.up_ch;
+                        reinterpret_cast<uint4*>(x.up)[at / 8 + c] = v;
+                    }
                 }
             }
             if (x.pool) {

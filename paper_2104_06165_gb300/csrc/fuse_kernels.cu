@@ -27,12 +27,15 @@
 //   agreement: ((e0 e0 + e1 e1) + e2 e2) < (tol d)^2 with e = X - X'
 //   point: (X + X'_b1 + X'_b2 + ...) / count, summed in view order.
 //
-// What bounds it: scattered reads of the later views and the launches of the
-// small views.  A view's depth and whether a pixel is still present share one
+// What bounds it: the latency of the gathers from the later views (the claim
+// pass of a 2048 x 1365 view issues in 54 % of its slots at 4 % of the DRAM's
+// rate; its warps wait for gathers and, at the count's barrier, for the slowest
+// warp of the block) and the launches of the small views.  A view's depth and whether a pixel is still present share one
 // compact float array (zero = absent), so that a gather touches 4 bytes of a
 // 32-byte sector that the neighbours use too instead of a flag and 4 of a
-// plane's 16 bytes; one launch prepares all views, the claim pass notes which views a pixel claimed
-// from, so that the merge projects into those only, and its blocks also count their pixels, the last of them to finish scanning the
+// plane's 16 bytes.  One launch prepares all views; the claim pass notes which
+// views a pixel claimed from, so that the merge projects into those only; its
+// blocks also count their pixels and the last of them to finish scans the
 // counts, so a view takes two launches instead of four (8 views, 13.5 M
 // pixels: 796 us against 1005).
 #include <algorithm>
@@ -66,7 +69,8 @@ __device__ __forceinline__ bool fuse_project(const FuseView& c, const float X[3]
                                    __fmul_rn(c.R[3 * k + 2], X[2])),
                          c.t[k]);
     if (!(q[2] > 0.0f)) return false;
-    const float u = __fdiv_rn(__fadd_rn(__fadd_rn(__fmul_rn(c.fx, q[0]), __fmul_rn(c.sk, q[1])), __fmul_rn(c.cx, q[2])), q[2]);
+    const float u = __fdiv_rn(__fadd_rn(__fadd_rn(__fmul_rn(c.fx, q[0]), __fmul_rn(c.sk, q[1])), __fmul_rn(c.cx, q[2])),
+                              q[2]);
     const float v = __fdiv_rn(__fadd_rn(__fmul_rn(c.fy, q[1]), __fmul_rn(c.cy, q[2])), q[2]);
     const float fu = floorf(__fadd_rn(u, 0.5f)), fv = floorf(__fadd_rn(v, 0.5f));
     if (!(fu >= 0.0f && fu <= (float)(c.W - 1) && fv >= 0.0f && fv <= (float)(c.H - 1))) return false;
@@ -122,7 +126,8 @@ __device__ __forceinline__ void fuse_scan(const int* block_count, long long* __r
 
 // pass 1: every present pixel of view a claims the pixels of later views it
 // agrees with (the lowest index wins, as in the raster-order statement) and
-// notes the views in `hits`; each block counts its present pixels and the last block to finish scans the counts
+// notes the views in `hits`; each block counts its present pixels and the last
+// block to finish scans the counts
 __global__ void __launch_bounds__(kFuseBlock) k_fuse_claim(const FuseView* __restrict__ views, int n, int a, float tol,
                                                            int* block_count, long long* __restrict__ block_off,
                                                            long long* __restrict__ total, unsigned* finished) {

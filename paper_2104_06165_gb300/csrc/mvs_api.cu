@@ -311,11 +311,21 @@ mvs_status ensure_map(mvs_ctx* c, int32_t v) {
 
 // The phases' workspace, one per context (its views run one after another):
 // the refinement perturbations of an iteration (20 bytes per pixel) and, when
-// the call visits every pixel often enough to pay for storing the windows (an
-// initialisation, which builds them anyway, or at least two iterations) and
-// workspace.h lets them have the memory, the stored windows; otherwise the phases rebuild each window, with
-// the same results.  One choice for all n views of a call, of at most
-// max_pixels pixels each and with the same window.
+// the call visits every pixel often enough to pay for storing the windows and
+// workspace.h lets them have the memory, the stored windows; otherwise the
+// phases rebuild each window, with the same results.  One choice for all n
+// views of a call, of at most max_pixels pixels each and with the same window.
+//
+// After an initialisation, which builds the windows anyway, one phase pays;
+// from a given state, whose windows k_window builds, it takes two iterations.
+// Stored against rebuilt, ms of a call with 10 sources and 11 x 11 samples:
+// initialisation and 1, 2, 4 phases 15.0 / 15.4, 23.9 / 25.1, 40.8 / 43.6 at
+// 1536 x 1024 and 70.3 / 69.6, 105.6 / 106.7, 171.7 / 179.3 at 3072 x 2048;
+// given state and 4, 8 phases 31.6 / 33.9, 54.2 / 59.7 and 150.6 / 155.3, 253.5
+// / 269.1.  k_window costs 0.9 and 6 ms there and a phase saves 0.8 and 2.7 ms,
+// so two phases from a given state would lose at the larger size.  A context
+// pays once for the memory, about 1 ms in its first call and 2.5 ms when it is
+// destroyed for the 6.9 GB of a 3072 x 2048 view.
 cudaError_t use_workspace(mvs_ctx* c, RefConst* rcs, int n, size_t max_pixels, const mvs_pm_params* p, int phases) {
     if (phases == 0) return cudaSuccess;
     const bool init = p->init_mode == MVS_INIT_RANDOM || p->init_mode == MVS_INIT_RANGE;
@@ -623,8 +633,8 @@ mvs_status mvs_patchmatch_batch(mvs_ctx* c, int32_t n_ref, const int32_t* refs, 
     BatchGraph* hit = nullptr;
     BatchGraph* lru = &c->batch[0];
     for (auto& b : c->batch) {
-        if (b.exec && b.refs == kr && b.srcs == ks && b.lanes == q.lanes_per_pixel && b.draws == rcs[0].draw4 && b.win == rcs[0].win &&
-            std::memcmp(&b.params, &q, sizeof q) == 0)
+        if (b.exec && b.refs == kr && b.srcs == ks && b.lanes == q.lanes_per_pixel && b.draws == rcs[0].draw4 &&
+            b.win == rcs[0].win && std::memcmp(&b.params, &q, sizeof q) == 0)
             hit = &b;
         if (!b.exec || (lru->exec && b.used < lru->used)) lru = &b;
     }
@@ -648,7 +658,8 @@ mvs_status mvs_patchmatch_batch(mvs_ctx* c, int32_t n_ref, const int32_t* refs, 
             else if (p->init_mode == MVS_INIT_GIVEN_RECOST)
                 e = launch_cost(rcs[r], rcs[r].plane, rcs[r].cost, nullptr, c->gstream);
             if (e == cudaSuccess) e = launch_memo_reset(rcs[r], c->gstream);
-            for (int ph = p->phase_begin; ph < pend && e == cudaSuccess; ++ph) e = launch_phase(rcs[r], ph, ph == p->phase_begin, c->gstream);
+            for (int ph = p->phase_begin; ph < pend && e == cudaSuccess; ++ph)
+                e = launch_phase(rcs[r], ph, ph == p->phase_begin, c->gstream);
         }
         cudaError_t e2 = cudaStreamEndCapture(c->gstream, &g);
         if (e == cudaSuccess) e = e2;

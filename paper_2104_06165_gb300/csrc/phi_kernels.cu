@@ -28,8 +28,9 @@ __device__ __forceinline__ void mat3v(const float* M, float a, float b, float c,
 // Memory-bound (71 % of the DRAM's rate): pixels of wrong depth project
 // anywhere, so the sources are read about three times.  A block is a 32 x 8
 // tile, so that the source pixels its projections share are in L1 whatever the
-// direction a source turns a row to (3072 x 2048, ten sources: 639 us in rows of
-// 256, 626 us in tiles; 16 x 16 the same, 8 x 32 643 us).
+// direction a source turns a row to.  That gives little (3072 x 2048, ten
+// sources, timed in turn: 647 us in rows of 256, 633 in tiles, about what runs
+// differ by; 16 x 16 the same, 8 x 32 slower than rows).
 constexpr int kGeoX = 32, kGeoY = 8;
 __global__ void __launch_bounds__(kGeoX * kGeoY) k_geo_filter(const __grid_constant__ FilterConst fc,
                                                               uint8_t* __restrict__ keep, int32_t* __restrict__ count) {
@@ -351,7 +352,8 @@ __global__ void __launch_bounds__(kBlock, S <= 9 ? 5 : S <= 11 ? 4 : 3)
 // tie).  A node depends on its up / left neighbours only (forward; on its down
 // / right ones in the backward pass, which runs the same schedule on the
 // mirrored grid), so the rows run as a pipeline with the messages of the
-// sequential sweep.
+// sequential sweep (up to rounding next to holes with one hypothesis, see
+// from_known).
 //
 // What bounds it: a chain of gw + gh - 1 dependent nodes.  One warp walks one
 // row, lane (d, lq, l) evaluating the min-sum term of own label l towards
@@ -537,9 +539,12 @@ __global__ void __launch_bounds__(32 * kTrwRows, 1) k_trw_rows(MrfBufs mb, bool 
         uint32_t f_info = 0;
         int f_lu = 0;
         // message to node i (L labels) from its pass-local upper (d 0) or left
-        // (d 1) neighbour q with one label: that neighbour's belief and the
-        // message into it are zero, so it is the pair energies less their
-        // minimum, whatever the pass; also stored for the other pass
+        // (d 1) neighbour q with one label: every label of i sees the same
+        // belief of q, which the normalisation takes out, so the message is
+        // the pair energies less their minimum, whatever the pass; also stored
+        // for the other pass.  For a reconstructed neighbour, whose belief is
+        // zero, that is the sweep's message bit for bit; a hole with a single
+        // hypothesis has a unary and messages, which cancel up to rounding.
         auto from_known = [&](long long i, long long q, int d, int L) {
             float v[4];
             if (forward) {
@@ -570,7 +575,8 @@ __global__ void __launch_bounds__(32 * kTrwRows, 1) k_trw_rows(MrfBufs mb, bool 
             f_lu = 0;
             const int L = labels(i);
             if (L >= 2) {
-                const long long qd = node(xf, yf + 1), qr = node(xf + 1, yf), qu = node(xf, yf - 1), ql = node(xf - 1, yf);
+                const long long qd = node(xf, yf + 1), qr = node(xf + 1, yf);
+                const long long qu = node(xf, yf - 1), ql = node(xf - 1, yf);
                 const int Ld = labels(qd), Lr = labels(qr), Lu = labels(qu), Ll = labels(ql);
                 const int mx = max((Lu > 0) + (Ll > 0), (Ld > 0) + (Lr > 0));
                 f_gm = mx > 0 ? 1.0f / (float)mx : 1.0f;
@@ -852,7 +858,8 @@ cudaError_t launch_geo_filter(const FilterConst& fc, uint8_t* keep, int32_t* cou
 }
 
 // Fixed line-map scratch of mvs_phi_hypotheses_static: 8 words per pixel (no
-// shape of an image needs more, see LineMaps) for up to MVS_PHI_STATIC_MAX_PIXELS pixels, in the library's own device memory.
+// shape of an image needs more, see LineMaps) for up to
+// MVS_PHI_STATIC_MAX_PIXELS pixels, in the library's own device memory.
 static __device__ __align__(256) int32_t g_phi_gaps_static[8 * (size_t)MVS_PHI_STATIC_MAX_PIXELS];
 
 // Device address of g_phi_gaps_static on the current device, looked up once
@@ -885,8 +892,8 @@ cudaError_t launch_phi_hypotheses(int W, int H, const float* depth, const uint8_
                                         (long long)lm.nwp * (W + H - 1)});
     k_line_bits<<<dim3(blocks_for(threads, 256), 4), 256, 0, s>>>(lm, known);
     count_launch();
-    k_line_sums<<<dim3(blocks_for(std::max<long long>(H, (long long)W + H - 1) * ((std::max(lm.nwx, (H + 31) / 32) + 31) / 32),
-                                  256), 4), 256, 0, s>>>(lm);
+    const long long sums = ((long long)W + H - 1) * ((std::max(lm.nwx, (H + 31) / 32) + 31) / 32);
+    k_line_sums<<<dim3(blocks_for(sums, 256), 4), 256, 0, s>>>(lm);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -920,7 +927,10 @@ cudaError_t launch_phi_cost(const RefConst& rc, const float* hyp, const uint8_t*
                             cudaStream_t s) {
     long long npix = (long long)((rc.W + step - 1) / step) * ((rc.H + step - 1) / step);
     const size_t smem = smem_block_bytes(rc.n_src, kWarps);
-#define CALL(G, S) k_phi_cost<G, S><<<pm_grid_for((const void*)k_phi_cost<G, S>, (npix + kWarps - 1) / kWarps, smem, kBlock), kBlock, smem, s>>>(rc, hyp, valid, hcost, step)
+    const long long units = (npix + kWarps - 1) / kWarps;
+#define CALL(G, S)                                                                                        \
+    k_phi_cost<G, S><<<pm_grid_for((const void*)k_phi_cost<G, S>, units, smem, kBlock), kBlock, smem, s>>>( \
+        rc, hyp, valid, hcost, step)
     MVS_DISPATCH(rc.n, CALL);
 #undef CALL
     count_launch();

@@ -560,10 +560,9 @@ struct PairGeo {
 //   CENTRED = true: sa += sum w (d - mean_d)^2.
 // The gathers run in chunks of up to 9 slots (registers).
 template <int G, int S, bool CENTRED, int CH = (S <= 9 ? S : (S + 1) / 2)>
-__device__ __forceinline__ void window_pass(const PixWin<S>& pw, int grp,
-                                            const uint2* __restrict__ tex, uint32_t pitch, uint32_t last,
-                                            const PairGeo& g, float nc0, float mean_d, float& sa, float& sb,
-                                            float& se) {
+__device__ __forceinline__ void window_pass(const PixWin<S>& pw, const uint2* __restrict__ tex, uint32_t pitch,
+                                            uint32_t last, const PairGeo& g, float nc0, float mean_d, float& sa,
+                                            float& sb, float& se) {
 #pragma unroll
     for (int k0 = 0; k0 < S; k0 += CH) {
         uint2 tq[CH];
@@ -820,7 +819,7 @@ __device__ __forceinline__ float eval_batch(const RefConst& rc, const ViewSm* __
         const uint2* v_tex = reinterpret_cast<const uint2*>(((unsigned long long)v0.y << 32) | v0.x);
         float sa = 0.0f, sb = 0.0f, se = 0.0f;
         if constexpr (!MIXED) {
-            window_pass<G, S, false>(pw, grp, v_tex, v0.z, v0.w, pg, nc0, 0.0f, sa, sb, se);
+            window_pass<G, S, false>(pw, v_tex, v0.z, v0.w, pg, nc0, 0.0f, sa, sb, se);
         } else {
             double unused = 0.0;
             window_pass_h2<G, S, 0>(pw, v_tex, v0.z, v0.w, pg, nc0, 0.0f, sa, sb, se, unused);
@@ -841,7 +840,7 @@ __device__ __forceinline__ float eval_batch(const RefConst& rc, const ViewSm* __
             const float md = __shfl_sync(0xffffffffu, mean_d, lane & ~(G - 1));
             float s2 = 0.0f, u0 = 0.0f, u1 = 0.0f;
             if constexpr (!MIXED) {
-                window_pass<G, S, true>(pw, grp, v_tex, v0.z, v0.w, pg, nc0, md, s2, u0, u1);
+                window_pass<G, S, true>(pw, v_tex, v0.z, v0.w, pg, nc0, md, s2, u0, u1);
             } else {
                 double unused = 0.0;
                 window_pass_h2<G, S, 1>(pw, v_tex, v0.z, v0.w, pg, nc0, md, s2, u0, u1, unused);

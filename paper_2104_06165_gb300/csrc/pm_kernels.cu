@@ -46,10 +46,16 @@ constexpr int kWarps = kBlock / 32;
 // 1139 with 16, 1239 with 32; 1511 x 1007 the same within 1 %), a vertical
 // one shares more L1 lines than a square (2 x 10: 4 % slower).
 constexpr int kTileY = 8;
-// Warps of the block: with the windows read back, 24 warps at 80 registers (a
-// few spilled outside the sample loop) hide more latency than 20 at 96 (1511 x
-// 1007, 8 iterations: 75.0 against 78.2 ms; 16 warps 78.6, 28 warps 75.5).
-// Layouts with more slots per lane need the registers.
+// Warps of the block: 24 at 80 registers (11 x 11 samples: 80 to 120 bytes
+// spilled outside the sample loop) were chosen with the windows read back and
+// an earlier sample loop (1511 x 1007, 8 iterations: 75.0 ms against 78.2 with
+// 20 at 96, 78.6 with 16, 75.5 with 28).  With this loop 20 are a little better
+// where the windows are read back (24 / 20 warps, timed in turn: 320 x 240 1058
+// / 1042 us, 1511 x 1007 76.3 / 75.6 ms, 3072 x 2048 383 / 367 ms, six views in
+// a batch 127.2 / 124.6 ms); where they are rebuilt (two phases from a given
+// state, 1536 x 1024, 24 / 20 / 16 warps) mixed precision takes 18.5 / 18.5 /
+// 19.0 ms and FP32 18.4 / 18.6 / 17.6.  Layouts with more slots per lane need
+// the registers.
 template <int S>
 constexpr int phase_max_warps() { return S <= 9 ? 24 : S <= 11 ? 20 : S <= 14 ? 16 : 12; }
 
@@ -132,8 +138,9 @@ __global__ void __launch_bounds__(kBlock, one_hyp_blocks<S>()) k_window(const __
 
 // cost of a given plane map
 template <int G, int S, bool MIXED>
-__global__ void __launch_bounds__(kBlock, one_hyp_blocks<S>()) k_cost(const __grid_constant__ RefConst rc, const float4* __restrict__ plane,
-                                                  float* __restrict__ cost, float* view_cost) {
+__global__ void __launch_bounds__(kBlock, one_hyp_blocks<S>())
+    k_cost(const __grid_constant__ RefConst rc, const float4* __restrict__ plane, float* __restrict__ cost,
+           float* view_cost) {
     extern __shared__ __align__(16) unsigned char smem[];
     ViewSm* views = reinterpret_cast<ViewSm*>(smem);
     load_views(rc, views);

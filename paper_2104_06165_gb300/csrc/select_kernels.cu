@@ -402,7 +402,7 @@ cudaError_t launch_sparse_range(int ref, int n_views, const double Rrow2[3], dou
     if (!all && (e = cudaMemsetAsync(cell_n, 0, (size_t)nc * sizeof(unsigned), s)) != cudaSuccess) return e;
     const unsigned long long views_mask = n_views >= 64 ? ~0ULL : ((1ULL << n_views) - 1ULL);
     if (n_pts > 0) {
-        const unsigned nb = (unsigned)std::min<long long>((n_pts + 255) / 256, 152LL * 8), np = (unsigned)((n_pts + 255) / 256);
+        const unsigned np = (unsigned)((n_pts + 255) / 256), nb = std::min(np, 152u * 8u);
         k_sparse_count<<<nb, 256, 0, s>>>(vis, n_pts, views_mask, total);
         k_sparse_features<<<np, 256, 0, s>>>(X, vis, reproj, obs, n_pts, views_mask, total, ref, Rrow2[0], Rrow2[1],
                                              Rrow2[2], t2, max_reproj, cell, ncx, ncy, feat, all ? nullptr : cell_of,
@@ -419,7 +419,8 @@ cudaError_t launch_sparse_range(int ref, int n_views, const double Rrow2[3], dou
     if (all)
         k_sparse_range_all<<<grid, kRangeTile * kRangeTile, 0, s>>>(feat, n_pts, W, H, d_lo, d_hi, range);
     else
-        k_sparse_range<<<grid, kRangeTile * kRangeTile, 0, s>>>(binned, cell_start, cell, ncx, ncy, W, H, d_lo, d_hi, range);
+        k_sparse_range<<<grid, kRangeTile * kRangeTile, 0, s>>>(binned, cell_start, cell, ncx, ncy, W, H, d_lo, d_hi,
+                                                                range);
     count_launch();
     return cudaGetLastError();
 }
