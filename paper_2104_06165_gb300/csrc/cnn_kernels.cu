@@ -330,7 +330,7 @@ __global__ void k_proposal_loss(const float* __restrict__ out, const float4* __r
         uint4 q[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
         if (mask[i]) {
             // the head's 16 outputs in 16-byte loads
-            float outv[16];
+            alignas(16) float outv[16];
 #pragma unroll
             for (int k = 0; k < 4; ++k) reinterpret_cast<float4*>(outv)[k] = reinterpret_cast<const float4*>(out)[4 * i + k];
             const float4 t4 = target[i];
