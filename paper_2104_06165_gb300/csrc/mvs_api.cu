@@ -301,10 +301,15 @@ mvs_status ensure_map(mvs_ctx* c, int32_t v) {
     ViewData& V = c->views[v];
     if (V.plane) return MVS_OK;
     size_t n = (size_t)V.cam.width * V.cam.height;
-    CK(c, ctx_malloc(c, &V.plane, n * sizeof(float4)));
-    CK(c, ctx_malloc(c, &V.cost, n * sizeof(float)));
-    CK(c, ctx_malloc(c, &V.memo, n * MVS_MEMO_WORDS * sizeof(uint32_t)));
-    CK(c, ctx_malloc(c, &V.gen, n * sizeof(uint32_t)));
+    const size_t bytes[4] = {n * sizeof(float4), n * sizeof(float), n * MVS_MEMO_WORDS * sizeof(uint32_t),
+                             n * sizeof(uint32_t)};
+    void* p[4];
+    CtxMemory mem{c};
+    if (!ws_get_all(c->work, bytes, p, 4, mem)) CK(c, mem.err);   // (the map is there whole or not at all)
+    V.plane = (float4*)p[0];
+    V.cost = (float*)p[1];
+    V.memo = (uint32_t*)p[2];
+    V.gen = (uint32_t*)p[3];
     CK(c, cudaMemsetAsync(V.gen, 0, n * sizeof(uint32_t), c->stream));
     return MVS_OK;
 }

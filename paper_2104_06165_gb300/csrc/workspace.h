@@ -45,6 +45,18 @@ void* ws_get(PhaseWorkspace& w, size_t bytes, A& a) {
     return p;
 }
 
+// n buffers, all or none.
+template <class A>
+bool ws_get_all(PhaseWorkspace& w, const size_t* bytes, void** p, int n, A& a) {
+    for (int i = 0; i < n; ++i) {
+        p[i] = ws_get(w, bytes[i], a);
+        if (p[i]) continue;
+        while (i > 0) a.put(p[--i]);
+        return false;
+    }
+    return true;
+}
+
 // Makes `draws` bytes and, when they can be had, `windows` bytes ready for one
 // call; false when the first cannot.  *stored: whether the windows are there.
 // The caller takes the two pointers once, for all views of the call.  A buffer

@@ -43,7 +43,7 @@ struct Fake {
 };
 // arguments: room, limit, then "draws windows" per call; draws < 0: that much
 // for something else of the context (-1: free bytes that cannot be had, -2:
-// whether the calls are captured)
+// whether the calls are captured, -3: a map of 2 x windows bytes in four buffers)
 int main(int argc, char** argv) {
     Fake a{(size_t)std::atoll(argv[1])};
     PhaseWorkspace w;
@@ -55,7 +55,12 @@ int main(int argc, char** argv) {
         if (d < 0) {
             if (d == -1) a.hidden = windows;
             if (d == -2) a.captures = windows != 0;
-            const bool got = d >= -2 || ws_get(w, -d, a) != nullptr;
+            bool got = d >= -2 || (d != -3 && ws_get(w, -d, a) != nullptr);
+            if (d == -3) {
+                const size_t b[4] = {windows, windows / 4, windows / 2, windows / 4};
+                void* p[4];
+                got = ws_get_all(w, b, p, 4, a);
+            }
             std::printf("%d 0 1 %d %d %d %zu %zu %zu\n", (int)got, a.gets, a.fails, a.puts, (size_t)w.draws.p,
                         (size_t)w.windows.p, a.used());
             continue;
@@ -140,6 +145,14 @@ def test_what_a_captured_call_uses_stays(workspace):
     # windows of a captured call give way to nothing
     r = workspace(2020, 1 << 40, (20, 0), (20, 900), (-2, 1), (20, 900), (-2, 0), (-1500, 0))
     assert [c[0] for c in r] == [1, 1, 1, 1, 1, 0] and r[5][7] == r[1][7]
+
+
+def test_a_map_is_there_whole_or_not_at_all(workspace):
+    r = workspace(1900, 1 << 40, (-3, 1000), (-3, 800))
+    assert [c[0] for c in r] == [0, 1] and [c[8] for c in r] == [0, 1600]
+    # windows give way to it
+    r = workspace(2000, 1 << 40, (20, 900), (-3, 800))
+    assert [c[0] for c in r] == [1, 1] and r[1][8] == 1620
 
 
 def test_limit_and_no_room_at_all(workspace):
