@@ -247,7 +247,7 @@ mvs_status mvs_plane_cost(mvs_ctx* ctx, int32_t ref, const int32_t* srcs, int32_
  *   min_consistent source maps, else 0; count (H*W int32, may be NULL)
  *   receives the number of consistent views.
  * Errors: MVS_ESTATE if ref or a source has no depth map in the context,
- *   MVS_EINVAL, MVS_ECUDA. */
+ *   MVS_EINVAL, MVS_ECUDA, MVS_ETIMEOUT (see mvs_plane_infer). */
 mvs_status mvs_geo_filter(mvs_ctx* ctx, int32_t ref, const int32_t* srcs, int32_t n_src,
                           const mvs_filter_params* fp, uint8_t* keep_mask, int32_t* count, int32_t mem);
 
@@ -279,7 +279,7 @@ mvs_status mvs_geo_filter(mvs_ctx* ctx, int32_t ref, const int32_t* srcs, int32_
  *   more points than capacity: then the first `capacity` points are written
  *   and *n_points holds the full count), MVS_ESTATE (a view without depth
  *   map), MVS_EUNSUPPORTED (a view whose K is not pinhole), MVS_ENOMEM,
- *   MVS_ECUDA. */
+ *   MVS_ECUDA, MVS_ETIMEOUT (see mvs_plane_infer). */
 mvs_status mvs_fuse(mvs_ctx* ctx, int32_t n_views, const int32_t* views, const uint8_t* const* keep_masks,
                     float rel_tol, float* points, int32_t* src, int64_t* owner, int64_t capacity,
                     int64_t* n_points, int32_t mem);
@@ -564,7 +564,8 @@ mvs_status mvs_cnn_propose(mvs_cnn* net, const uint8_t* img, const float* plane,
 /* mvs_cnn_propose on the image and the current depth map of context view
  * `ref` (the state left by the last mvs_patchmatch of that view); runs on
  * the context stream, which must be the network's device.
- * Errors: MVS_ESTATE if the view has no map, MVS_EINVAL, MVS_ECUDA. */
+ * Errors: MVS_ESTATE if the view has no map, MVS_EINVAL, MVS_ECUDA,
+ *   MVS_ETIMEOUT (see mvs_plane_infer). */
 mvs_status mvs_propose(mvs_ctx* ctx, int32_t ref, mvs_cnn* net, float* proposals);
 
 #ifdef __cplusplus
